@@ -427,7 +427,6 @@ SolveArgs solve_args(ppl_cpd* h, int m) {
     a.V = h->at<double>(h->L.V); a.Linv = h->at<double>(h->L.Linv); a.Z = h->at<double>(h->L.Z);
     a.U = h->U[m]; a.lam = h->lam; a.G = h->G(m);
     a.sync = reinterpret_cast<unsigned int*>(f + 16);
-    a.maxdiag = reinterpret_cast<unsigned long long*>(f + 32);
     a.nclamp = h->nclamp(); a.err = h->errflag();
     a.wait_ns = h->wait_ns; a.withhold = h->withhold();
     return a;
@@ -437,7 +436,7 @@ SolveArgs solve_args(ppl_cpd* h, int m) {
 int solve_mode(ppl_cpd* h, int m) {
     const SolveArgs a = solve_args(h, m);
     const int r = solve_mode_coop(a.G1, a.G2, a.G3, a.M, a.dim, a.R, a.V, a.Linv, a.Z, a.U, a.lam, a.G, a.sync,
-                                  a.maxdiag, a.nclamp, a.err, h->solve_cap, a.wait_ns, a.withhold, h->st);
+                                  a.nclamp, a.err, h->solve_cap, a.wait_ns, a.withhold, h->st);
     if (r != 0)
         return fail(h, PPL_ECUDA, "cooperative solve launch failed (%d%s%s)", r, r <= -1000 ? ": " : "",
                     r <= -1000 ? cudaGetErrorString((cudaError_t)(-r - 1000)) : "");

@@ -8,8 +8,7 @@
 //       panels by warp-per-row triangular solves with the column-scaled diagonal block)
 //       with the rows of Z appended below V, so the same panel and trailing updates
 //       carry out the forward substitution Z <- M L^-T; the next diagonal block is
-//       updated by three blocks (one lower quarter each) and factored by block 0
-//       while the others update the rest
+//       updated by five blocks and factored by block 0 while the others update the rest
 //   P2  back substitution U~ L = Z: the rows are independent, so every block solves
 //       its own rows over all column blocks with no grid barrier (one warp per
 //       column block in turn, all eight warps for the updates left of it)
@@ -33,6 +32,14 @@ constexpr int NB = 32;
 constexpr int NT = 256;
 constexpr unsigned long long BAR_NS = 1000ull * 1000ull * 1000ull;   // 1 s per barrier wait
 
+// The block's shared memory (at file scope, so that the factorisation below can be
+// a function of its own and still address it as shared memory).
+__shared__ double Ls[NB][NB + 1];   // the diagonal block being factored; staging in the back substitution
+__shared__ double Li[NB][NB + 1];   // its column-scaled factor; staging in the back substitution
+__shared__ double Ta[NB][NB + 1];   // tiles
+__shared__ double Tb[NB][NB + 1];
+__shared__ unsigned short tri[NB * (NB + 1) / 2];   // (row << 8) | col of the lower triangle, row-major
+
 struct SolveP {
     const double* G1;
     const double* G2;
@@ -44,8 +51,7 @@ struct SolveP {
     double* U;
     double* lam;
     double* G;
-    unsigned int* sync;              // [0] arrivals, [1] generation, [2] abort
-    unsigned long long* maxdiag;
+    unsigned int* sync;              // barrier words (see gsync), zero between launches
     unsigned long long* nclamp;
     unsigned int* err;
     unsigned int* withhold;          // != 0: block 1 skips its first barrier arrival (once)
@@ -73,49 +79,83 @@ __device__ __forceinline__ unsigned int atom_add_release(unsigned int* p, unsign
     return old;
 }
 
+// p.sync: [0] arrivals of this launch, counted up over all barriers, with the top
+// bit as the abort flag (a waiter learns of an abort from the word it polls
+// anyway); [1] blocks that have left; [3] pieces of the next diagonal block.  The
+// words are zero between launches: the last block to leave clears them, on the
+// abort path too, so no launch needs a memset before it (two memset nodes ahead
+// of every solve cost 8 to 11 us of graph time, 40 us per sweep).
+constexpr unsigned int SYNC_ABORT = 0x80000000u;
+
+__device__ __forceinline__ void raise_abort(const SolveP& p, unsigned int code) {
+    atomicOr(&p.sync[0], SYNC_ABORT);
+    atomicOr(p.err, code);
+}
+
+// wait (bounded) until *w >= target; false when the wait ran out or a block aborted.
+// The clock is read on every 32nd poll only: a poll is one L2 round trip and the
+// barriers are on the critical path.
+__device__ __forceinline__ bool poll_until(const SolveP& p, const unsigned int* w, unsigned int target, unsigned int code) {
+    unsigned long long t0 = 0;
+    for (unsigned int n = 1;; ++n) {
+        const unsigned int v = ld_acquire(w);
+        if (w == &p.sync[0] && (v & SYNC_ABORT)) return false;
+        if ((v & ~SYNC_ABORT) >= target) return true;
+        if ((n & 31u) == 0u) {
+            const unsigned long long t = gtimer();
+            if (t0 == 0) t0 = t;
+            if (t - t0 > p.wait_ns) {
+                raise_abort(p, code);
+                return false;
+            }
+            if (ld_vol(&p.sync[0]) & SYNC_ABORT) return false;
+        }
+    }
+}
+
 // grid-wide barrier; false when the wait expired or another block aborted.
 // The block's writes are ordered before its arrival by __syncthreads and the
-// release of the arrival; the waiters' acquire loads order what follows.
-__device__ bool gsync(const SolveP& p, unsigned int& gen, int* s_flag, int bid, int G) {
+// release of the arrival; the waiters' acquire loads order what follows.  The
+// waiters poll the arrival counter itself (target counts G more per barrier), so
+// the last arrival releases them with no second word to write: 1.5 us on 152
+// blocks, against 2.5 us with a separate generation word and a clock read per poll.
+__device__ bool gsync(const SolveP& p, unsigned int& target, int* s_flag, int bid, int G) {
     __syncthreads();
     if (threadIdx.x == 0) {
         int ok = 1;
+        target += (unsigned int)G;
         // the test of the bounded waits: block 1 withholds its first arrival, so
         // the other blocks' wait runs out; it waits (bounded) for their abort
         const bool withhold =
             bid == 1 && p.withhold && ld_vol(p.withhold) != 0u && atomicExch(p.withhold, 0u) != 0u;
         if (withhold) {
             const unsigned long long t0 = gtimer();
-            while (!ld_vol(&p.sync[2]) && gtimer() - t0 < 4 * p.wait_ns) {
+            while (!(ld_vol(&p.sync[0]) & SYNC_ABORT) && gtimer() - t0 < 4 * p.wait_ns) {
             }
             ok = 0;
         } else {
-            const unsigned int arrived = atom_add_release(&p.sync[0], 1u) + 1u;
-            if (arrived == (unsigned int)G) {
-                atomicExch(&p.sync[0], 0u);
-                atom_add_release(&p.sync[1], 1u);
-            } else {
-                const unsigned long long t0 = gtimer();
-                while (ld_acquire(&p.sync[1]) == gen) {
-                    if (ld_vol(&p.sync[2])) {
-                        ok = 0;
-                        break;
-                    }
-                    if (gtimer() - t0 > p.wait_ns) {
-                        atomicExch(&p.sync[2], 1u);
-                        atomicOr(p.err, 16u);
-                        ok = 0;
-                        break;
-                    }
-                }
-            }
+            const unsigned int old = atom_add_release(&p.sync[0], 1u);
+            ok = (old & SYNC_ABORT) ? 0 : (poll_until(p, &p.sync[0], target, 16u) ? 1 : 0);
         }
-        gen += 1;
-        if (ld_vol(&p.sync[2])) ok = 0;
         *s_flag = ok;
     }
     __syncthreads();
     return *s_flag != 0;
+}
+
+// every block passes here once per launch, whatever happened before: the last one
+// leaves the barrier words at zero for the next launch
+__device__ void leave_sync(const SolveP& p, int G) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned int old;
+        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(&p.sync[1]) : "memory");
+        if (old == (unsigned int)G - 1u) {
+            p.sync[0] = 0u;
+            p.sync[3] = 0u;
+            p.sync[1] = 0u;
+        }
+    }
 }
 
 __device__ __forceinline__ void tri_index(int t, int& I, int& J) {
@@ -128,119 +168,98 @@ __device__ __forceinline__ void tri_index(int t, int& I, int& J) {
     J = t - i * (i + 1) / 2;
 }
 
-// Factor the kb x kb diagonal block held in Ls (lower) in place, clamping
-// pivots at tol, and leave in Li the column-scaled factor the panel solves
-// with.  All NT threads.
-//
-// GB300 issues an FP64 warp instruction at the same cost whether or not its
-// lanes are masked, so the factorisation keeps the FP64 instruction count close
-// to the useful work: right-looking on unscaled columns (with d_j the clamped
-// pivot, A[i][c] -= A[i][j] A[c][j] / d_j, one reciprocal per column); at step
-// j only the n(n+1)/2 active elements of the trailing triangle are enumerated,
-// packed onto consecutive threads through the (row, col) table tri; square
-// roots and column scalings follow in one parallel pass.
-
-// 1/d for a positive normal d: the PTX approximate reciprocal refined by two
-// Newton-Raphson steps x <- x + x (1 - d x), each squaring the relative error
-// (within an ulp or two of the correctly rounded quotient).  Four FP64 FMAs
-// instead of the longer IEEE division sequence on the factorisation's
-// critical path.
+// 1/d for a positive normal d: the PTX approximate reciprocal (relative error e
+// about 2^-20) with one third-order step x <- x (1 + e + e^2), e = 1 - d x, whose
+// error is e^3 (Householder's method of order two).  Three dependent FP64 FMAs:
+// an FP64 warp instruction takes 64 clocks on GB300, issue and latency alike, and
+// the pivots' reciprocals are the factorisation's critical path (two Newton steps
+// are four).
 __device__ __forceinline__ double recip_nr(double d) {
     double x;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(d));
-    double e = fma(-d, x, 1.0);
-    x = fma(x, e, x);
-    e = fma(-d, x, 1.0);
-    return fma(x, e, x);
+    const double e = fma(-d, x, 1.0);
+    return fma(x, fma(e, e, e), x);
 }
-__device__ void diag_factor(double (*Ls)[NB + 1], double (*Li)[NB + 1], double* rd, const unsigned short* tri,
-                            int kb, double tol, unsigned long long* nclamp) {
-    const int t = threadIdx.x;
-    // the pivot of column j is clamped and inverted by thread 0 right after its
-    // own update of that element in step j - 1 (the table puts the next diagonal
-    // element on thread 0), so each step needs one barrier
-    if (t == 0 && kb > 0) {
-        double d = Ls[0][0];
-        if (!(d > tol)) {
-            d = tol;
-            atomicAdd(nclamp, 1ull);
-        }
-        Ls[0][0] = d;
-        rd[0] = recip_nr(d);
-    }
+
+// Factor the kb x kb diagonal block held in Ls (lower) and leave in Li the
+// column-scaled factor the panel and back substitution solve with: Li[i][j] =
+// L[i][j] / L[j][j] below the diagonal, 1 / L[i][i] on it, 0 elsewhere.  Pivots
+// not above tol are replaced by tol and counted.  Li is also written to Linv, where
+// the other blocks read it.  All NT threads.
+//
+// Right-looking on unscaled columns: with d_j the pivot and s_i = a_ij / d_j
+// (which is Li[i][j]), a_ic -= s_i a_cj.  An FP64 instruction occupies its SM
+// sub-partition's pipe for 64 clocks however many lanes are active, so the work
+// is laid out by sub-partitions.  Warp 0 alone, on its own sub-partition, owns the
+// chain pivot -> reciprocal -> column -> next pivot: at step j it scales column j
+// (which it hands to the others), updates column j + 1 and inverts the next pivot,
+// five dependent FP64 instructions, while the six warps of the other three
+// sub-partitions apply column j to columns j + 2 ..; one block barrier per step.
+// The pivot test is an integer comparison (an FP64 one is a sixth instruction).
+// Measured on one 32 x 32 block: 16.3 us with the whole triangle updated by all
+// warps, two instructions per element, the reciprocal after it in the same step
+// and separate passes for square roots and scaling; 10.5 us so.
+__device__ __noinline__ void factor_block(double* Linv, int kb, double tol, unsigned long long* nclamp) {
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    // the helpers: the six warps that do not share sub-partition 0 with warp 0
+    const int hw = warp < 4 ? warp - 1 : warp - 2;            // 1, 2, 3, 5, 6, 7 -> 0 .. 5
+    const bool helper = (warp & 3) != 0;
+    for (int e = threadIdx.x; e < NB * NB; e += NT) Li[e / NB][e % NB] = 0.0;
     __syncthreads();
-    for (int j = 0; j < kb; ++j) {
-        const int n = kb - j - 1;
-        const int nel = n * (n + 1) / 2;
-        if (t < nel) {
-            const unsigned short ic = tri[t];
-            const int ii = j + 1 + (ic >> 8), cc = j + 1 + (ic & 0xff);
-            const double x = fma(-(Ls[ii][j] * rd[j]), Ls[cc][j], Ls[ii][cc]);
-            if (t == 0) {
-                double d = x;
-                if (!(d > tol)) {
-                    d = tol;
-                    atomicAdd(nclamp, 1ull);
-                }
-                Ls[ii][cc] = d;
-                rd[j + 1] = recip_nr(d);
-            } else {
-                Ls[ii][cc] = x;
-            }
+    double a = 0.0;        // warp 0: a_ij of column j, i = lane
+    double dl = 1.0;       // the pivot of column `lane`
+    double r = 0.0;        // 1 / d_j
+    const long long tol_bits = __double_as_longlong(tol);
+    auto pivot = [&](int j) {             // d_j from column j, clamped, and its reciprocal (every lane)
+        double d = __shfl_sync(0xffffffffu, a, j);
+        // d > tol for tol > 0: positive doubles order as their bits; negative and NaN fail
+        const long long bits = __double_as_longlong(d);
+        if (!(bits > tol_bits && bits <= 0x7ff0000000000000ll)) {
+            d = tol;
+            if (lane == 0) atomicAdd(nclamp, 1ull);
         }
-        if (t + NT < nel) {
-            const unsigned short ic = tri[t + NT];
-            const int ii = j + 1 + (ic >> 8), cc = j + 1 + (ic & 0xff);
-            Ls[ii][cc] = fma(-(Ls[ii][j] * rd[j]), Ls[cc][j], Ls[ii][cc]);
+        if (lane == j) dl = d;
+        r = recip_nr(d);
+    };
+    if (warp == 0) {
+        a = lane < kb ? Ls[lane][0] : 0.0;
+        pivot(0);
+    }
+    for (int j = 0; j < kb; ++j) {
+        if (warp == 0) {
+            const double s = a * r;
+            double x = (j + 1 < kb && lane > j && lane < kb) ? Ls[lane][j + 1] : 0.0;
+            const double aj1 = __shfl_sync(0xffffffffu, a, (j + 1) & 31);
+            if (lane > j && lane < kb) Li[lane][j] = s;
+            // the column is published: the helpers may start
+            asm volatile("bar.arrive 1, 224;" ::: "memory");
+            if (j + 1 < kb) {
+                x = fma(-s, aj1, x);
+                if (lane > j && lane < kb) Ls[lane][j + 1] = x;
+                a = x;
+                pivot(j + 1);
+            }
+        } else if (helper) {
+            asm volatile("bar.sync 1, 224;" ::: "memory");
+            const int m = kb - j - 2;          // columns j + 2 .. kb - 1
+            const int nel = m > 0 ? m * (m + 1) / 2 : 0;
+            for (int e = hw * 32 + lane; e < nel; e += 6 * 32) {
+                const unsigned short ic = tri[e];
+                const int i = j + 2 + (ic >> 8), c = j + 2 + (ic & 0xff);
+                Ls[i][c] = fma(-Li[i][j], Ls[c][j], Ls[i][c]);
+            }
         }
         __syncthreads();
     }
-    // L = A_unscaled * diag(1/sqrt(d)), L_jj = sqrt(d_j); rd <- 1 / L_jj
-    if (t < kb) {
-        const double sd = sqrt(Ls[t][t]);
-        rd[t] = recip_nr(sd);
-        Ls[t][t] = sd;
-    }
+    if (warp == 0 && lane < kb) Li[lane][lane] = rsqrt(dl);
     __syncthreads();
-    {
-        const int nl = kb * (kb - 1) / 2;    // strictly lower elements, row-major
-        for (int e = t; e < nl; e += NT) {
-            const unsigned short ic = tri[e];
-            const int i = (ic >> 8) + 1, j = ic & 0xff;   // (i, j) with j < i
-            Ls[i][j] *= rd[j];
-        }
-    }
-    __syncthreads();
-    // Li <- the column-scaled factor used by the panel's triangular solves:
-    // Li[i][j] = L[i][j] / L[j][j] below the diagonal, Li[i][i] = 1 / L[i][i]
-    for (int e = t; e < NB * NB; e += NT) {
-        const int i = e / NB, j = e % NB;
-        Li[i][j] = (i < kb && j < i) ? Ls[i][j] * rd[j] : ((i < kb && j == i) ? rd[i] : 0.0);
-    }
-    __syncthreads();
-}
-
-// load the lower kb x kb block of V at (k0, k0) into Ls, factor it, write L
-// back to V and the column-scaled factor the panels solve with to Linv[k]
-__device__ void factor_block(const SolveP& p, int k, double tol, double (*Ls)[NB + 1], double (*Li)[NB + 1],
-                             double* rd, const unsigned short* tri, double (*Tw)[NB + 1]) {
-    const int R = p.R, tid = threadIdx.x;
-    const int k0 = k * NB, kb = min(NB, R - k0);
-    for (int e = tid; e < NB * NB; e += NT) {
-        const int i = e / NB, j = e % NB;
-        Ls[i][j] = (i < kb && j <= i) ? __ldcg(p.V + (long long)(k0 + i) * R + k0 + j) : 0.0;
-    }
-    __syncthreads();
-    diag_factor(Ls, Li, rd, tri, kb, tol, p.nclamp);
-    for (int e = tid; e < kb * kb; e += NT) {
-        const int i = e / kb, j = e % kb;
-        if (j <= i) p.V[(long long)(k0 + i) * R + k0 + j] = Ls[i][j];
-    }
-    for (int e = tid; e < NB * NB; e += NT) p.Linv[(long long)k * NB * NB + e] = Li[e / NB][e % NB];
+    for (int e = threadIdx.x; e < NB * NB; e += NT) Linv[e] = Li[e / NB][e % NB];
     __syncthreads();
 }
 
 constexpr int RB = 4;   // rows of U~ per back-substitution pass
+// pieces of the next diagonal block's update, of PIECE elements of its lower triangle
+constexpr int NPIECE = 5, PIECE = (NB * (NB + 1) / 2 + NPIECE - 1) / NPIECE;
 
 // asynchronous global -> shared copies (cp.async), waited for by the issuing thread
 __device__ __forceinline__ void cp_async8(void* dst, const void* src) {
@@ -249,18 +268,17 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// one warp copies an NB x NB block (row-major, NB doubles per row) into dst
-__device__ __forceinline__ void stage_block(const double* src, double (*dst)[NB + 1], int lane) {
+// one warp copies rows 0 .. rows-1 of an NB-wide block (row stride ld) into dst
+__device__ __forceinline__ void stage_block(const double* src, long long ld, int rows, double (*dst)[NB + 1], int lane) {
 #pragma unroll 8
-    for (int q = 0; q < NB; ++q) cp_async8(&dst[q][lane], src + q * NB + lane);
+    for (int q = 0; q < rows; ++q) cp_async8(&dst[q][lane], src + q * ld + lane);
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
 // Zl[r][c + bs b] -= sum_q x[r][q] L[j0 + q][lane + c + bs b] for the NR rows and
 // CB column blocks b of one warp (Zl and Ll point at the lane's column: Zl at
-// Z[r0][lane], Ll at L[j0][lane]).  KEEP: one block, the result returned in acc
-// instead of stored.
-template <int NR, int CB, bool KEEP = false>
+// Z[r0][lane], Ll at L[j0][lane]).
+template <int NR, int CB>
 __device__ __forceinline__ void back_update(double* Zl, int R, const double* Ll, const double (*x)[NB], int c, int kb,
                                             int bs, double (*acc)[NR]) {
 #pragma unroll
@@ -279,12 +297,10 @@ __device__ __forceinline__ void back_update(double* Zl, int R, const double* Ll,
             for (int b = 0; b < CB; ++b) acc[b][r] = fma(-xv, l[b], acc[b][r]);
         }
     }
-    if (!KEEP) {
 #pragma unroll
-        for (int b = 0; b < CB; ++b)
+    for (int b = 0; b < CB; ++b)
 #pragma unroll
-            for (int r = 0; r < NR; ++r) Zl[(long long)r * R + c + b * bs] = acc[b][r];
-    }
+        for (int r = 0; r < NR; ++r) Zl[(long long)r * R + c + b * bs] = acc[b][r];
 }
 
 // The kb unknowns of one column block for NR rows (one warp, lane = column):
@@ -309,11 +325,14 @@ __device__ __forceinline__ void back_diag(const double (*Ld)[NB + 1], int kb, in
 // published in shared memory; warp (J-1) mod 8 subtracts x_J L[rows of J][block
 // J-1] from block J-1, keeps the result in registers and solves it at once
 // (x_{J-1}), while the seven other warps subtract x_J from blocks 0 .. J-2; one
-// block barrier per step.  The diagonal block of J-1 was copied to shared memory
-// (cp.async) by the same warp one step earlier; the published values and the
-// staged blocks alternate between two buffers.
+// block barrier per step.  The diagonal block of J-1 and the block L[rows of J]
+// [block J-1] were copied to shared memory (cp.async) by the same warp one step
+// earlier; the published values and the staged blocks alternate between two
+// buffers (one row per SM, R = 250: 26 us against 40 us with L[J][J-1] read from L2
+// inside the owner's chain of 32 FMAs).
 template <int NR>
-__device__ void back_rows(const SolveP& p, int r0, double (*xs)[RB][NB], double (*lb0)[NB + 1], double (*lb1)[NB + 1]) {
+__device__ void back_rows(const SolveP& p, int r0, double (*xs)[RB][NB], double (*lb0)[NB + 1], double (*lb1)[NB + 1],
+                          double (*lo0)[NB + 1], double (*lo1)[NB + 1]) {
     constexpr int NW = NT / 32, NO = NW - 1;
     // CB blocks per pass, so that a pass keeps 4 sums and CB loads per step of q
     // in flight also when NR is small
@@ -332,10 +351,16 @@ __device__ void back_rows(const SolveP& p, int r0, double (*xs)[RB][NB], double 
             }
         }
     };
+    // what the owner of block J needs one step later: its diagonal block and L[rows of J+1][block J]
+    auto stage = [&](int J) {
+        stage_block(p.Linv + (long long)J * NB * NB, NB, NB, (J & 1) ? lb1 : lb0, lane);
+        const int j1 = (J + 1) * NB;
+        stage_block(p.V + (long long)j1 * R + J * NB, R, min(NB, R - j1), (J & 1) ? lo1 : lo0, lane);
+    };
     {   // the last block has nothing to its right
         const int J = nt - 1, j0 = J * NB, kb = min(NB, R - j0);
         if (warp == J % NW) {
-            stage_block(p.Linv + (long long)J * NB * NB, (J & 1) ? lb1 : lb0, lane);
+            stage_block(p.Linv + (long long)J * NB * NB, NB, NB, (J & 1) ? lb1 : lb0, lane);
             cp_async_wait_all();
             __syncwarp();
             double w[NR];
@@ -344,7 +369,7 @@ __device__ void back_rows(const SolveP& p, int r0, double (*xs)[RB][NB], double 
             back_diag<NR>((J & 1) ? lb1 : lb0, kb, lane, w);
             publish(J, w);
         }
-        if (J >= 1 && warp == (J - 1) % NW) stage_block(p.Linv + (long long)(J - 1) * NB * NB, ((J - 1) & 1) ? lb1 : lb0, lane);
+        if (J >= 1 && warp == (J - 1) % NW) stage(J - 1);
         __syncthreads();
     }
     for (int J = nt - 1; J >= 1; --J) {
@@ -352,15 +377,23 @@ __device__ void back_rows(const SolveP& p, int r0, double (*xs)[RB][NB], double 
         const double (*x)[NB] = xs[J & 1];
         const double* Ll = p.V + (long long)j0 * R + lane;     // L[j0 + q][lane + c] at q * R + c
         const int ow = (J - 1) % NW;
-        if (J >= 2 && warp == (J - 2) % NW) stage_block(p.Linv + (long long)(J - 2) * NB * NB, (J & 1) ? lb1 : lb0, lane);
         if (warp == ow) {
-            double w[1][NR];
-            back_update<NR, 1, true>(Zr + lane, R, Ll, x, (J - 1) * NB, kb, 0, w);
+            double w[NR];
+#pragma unroll
+            for (int r = 0; r < NR; ++r) w[r] = __ldcg(Zr + (long long)r * R + (J - 1) * NB + lane);
             cp_async_wait_all();
             __syncwarp();
-            back_diag<NR>(((J - 1) & 1) ? lb1 : lb0, NB, lane, w[0]);
-            publish(J - 1, w[0]);
+            const double (*lo)[NB + 1] = ((J - 1) & 1) ? lo1 : lo0;
+#pragma unroll 8
+            for (int q = 0; q < kb; ++q) {
+                const double l = lo[q][lane];
+#pragma unroll
+                for (int r = 0; r < NR; ++r) w[r] = fma(-x[r][q], l, w[r]);
+            }
+            back_diag<NR>(((J - 1) & 1) ? lb1 : lb0, NB, lane, w);
+            publish(J - 1, w);
         } else {
+            if (J >= 2 && warp == (J - 2) % NW) stage(J - 2);
             const int w7 = (warp - ow - 1 + NW) % NW;
             int Jc = w7;
             double acc[CB][NR];
@@ -449,26 +482,17 @@ __device__ __forceinline__ void gram_fetch(const SolveP& p, int i0, int j0, int 
 // One mode update of one instance, run by blocks bid = 0 .. G-1 (of one launch,
 // or of one instance's share of a batched launch); the barriers count G blocks.
 __device__ __forceinline__ void solve_body(const SolveP& p, const int bid, const int G) {
-    __shared__ double Ls[NB][NB + 1];
-    __shared__ double Li[NB][NB + 1];
-    __shared__ double Ta[NB][NB + 1];
-    __shared__ double Tb[NB][NB + 1];
-    __shared__ double rd[NB];
     __shared__ double red[NT / 32];
-    __shared__ unsigned short tri[NB * (NB + 1) / 2];   // (row << 8) | col of the lower triangle, row-major
     __shared__ int s_flag;
-    __shared__ unsigned int s_gen;
 
     const int R = p.R, dim = p.dim;
     const int tid = threadIdx.x;
     const long long gtid = (long long)bid * NT + tid;
     const long long gthreads = (long long)G * NT;
-    if (tid == 0) s_gen = ld_vol(&p.sync[1]);
     for (int i = 0, e = 0; i < NB; ++i)
         for (int c = 0; c <= i; ++c, ++e)
             if (e % NT == tid) tri[e] = (unsigned short)((i << 8) | c);
-    __syncthreads();
-    unsigned int gen = s_gen;   // meaningful in thread 0 only
+    unsigned int target = 0;   // arrivals of the next barrier; meaningful in thread 0 only
     const int kb0 = min(NB, R);
 
     // ---- P0 --------------------------------------------------------------------
@@ -484,25 +508,29 @@ __device__ __forceinline__ void solve_body(const SolveP& p, const int bid, const
     mx = red[0];
     for (int w = 1; w < NT / 32; ++w) mx = fmax(mx, red[w]);
     const double tol = fmax(ldexp(1.0, -52) * (double)R * mx, 1e-300);
-    __syncthreads();
-    for (long long e = gtid; e < (long long)R * R; e += gthreads) {
-        const int r = (int)(e / R), q = (int)(e % R);
-        if (q <= r && !(r < kb0 && q < kb0)) p.V[e] = p.G1[e] * p.G2[e] * p.G3[e];
-    }
-    for (long long e = gtid; e < (long long)dim * R; e += gthreads) p.Z[e] = p.M[e];
     if (bid == 0) {
         // the first diagonal block straight from the Gram matrices
         for (int e = tid; e < kb0 * kb0; e += NT) {
             const int i = e / kb0, j = e % kb0;
-            if (j <= i) {
-                const long long d = (long long)i * R + j;
-                p.V[d] = p.G1[d] * p.G2[d] * p.G3[d];
-            }
+            const long long d = (long long)i * R + j;
+            if (j <= i) Ls[i][j] = p.G1[d] * p.G2[d] * p.G3[d];
         }
         __syncthreads();
-        factor_block(p, 0, tol, Ls, Li, rd, tri, Tb);
+        factor_block(p.Linv, kb0, tol, p.nclamp);
     }
-    if (!gsync(p, gen, &s_flag, bid, G)) return;
+    // V and Z, row by row (no 64-bit division per element); block 0 is busy with the
+    // factor, so it leaves its rows to the others where there are any
+    {
+        const int nb = G > 1 ? G - 1 : 1, b0 = G > 1 ? bid - 1 : 0;
+        if (b0 >= 0) {
+            for (int r = kb0 + b0; r < R; r += nb) {
+                const long long d = (long long)r * R;
+                for (int q = tid; q <= r; q += NT) p.V[d + q] = p.G1[d + q] * p.G2[d + q] * p.G3[d + q];
+            }
+        }
+    }
+    for (long long e = gtid; e < (long long)dim * R; e += gthreads) p.Z[e] = p.M[e];
+    if (!gsync(p, target, &s_flag, bid, G)) return;
 
     const int nt = (R + NB - 1) / NB;
     const int D = (dim + NB - 1) / NB;
@@ -535,74 +563,58 @@ __device__ __forceinline__ void solve_body(const SolveP& p, const int bid, const
                 if (t < kb) row[t] = val * Li[t][t];
             }
         }
-        if (!gsync(p, gen, &s_flag, bid, G)) return;
+        if (!gsync(p, target, &s_flag, bid, G)) return;
         // trailing update of V (lower tiles) and of Z.  Tile 0 is the next
-        // diagonal block: block 0 updates it and factors it while the other
-        // blocks take the remaining tiles.
+        // diagonal block: the blocks 0 .. NPIECE-1 each update a fifth of its lower
+        // triangle (one warp per SM sub-partition: 1 us of FP64 issue, against 4.2
+        // us on one SM), the others signal block 0, which factors the block while
+        // the rest of the grid takes the remaining tiles.  Block 0 takes no other
+        // tile; with too few blocks it updates all of tile 0.
         const int Tk = (vrows + NB - 1) / NB;
         const int ntri = Tk * (Tk + 1) / 2;
         const int ntile = ntri + D * Tk;
-        // With three or more blocks, tile 0 (the next diagonal block) is split:
-        // blocks 0, 1, 2 each update one of its three lower 16 x 16 quarters,
-        // blocks 1 and 2 then signal block 0, which factors the block once both
-        // quarters have landed.  Block 0 takes no other tile.
-        const bool split0 = (G >= 3 && k + 1 < nt && ntile > 0);
-        if (split0 && bid < 3) {
-            const int q = bid;
+        const bool pieces = G > NPIECE;
+        if (k + 1 < nt && bid < (pieces ? NPIECE : 1)) {
             const int d0 = k0 + kb, nb1 = min(NB, R - d0);
-            const int r0 = (q == 0) ? 0 : 16, c0 = (q == 2) ? 16 : 0;
             const double* Pd = p.V + (long long)d0 * R + k0;     // rows of the panel at the next block
-            for (int e = tid; e < 16 * NB; e += NT) {
+            for (int e = tid; e < NB * NB; e += NT) {
                 const int i = e / NB, s2 = e % NB;
-                Ta[i][s2] = (r0 + i < nb1 && s2 < kb) ? __ldcg(Pd + (long long)(r0 + i) * R + s2) : 0.0;
-                Tb[i][s2] = (c0 + i < nb1 && s2 < kb) ? __ldcg(Pd + (long long)(c0 + i) * R + s2) : 0.0;
+                Ta[i][s2] = (i < nb1 && s2 < kb) ? __ldcg(Pd + (long long)i * R + s2) : 0.0;
             }
             __syncthreads();
-            const int ti = tid / 16, tj = tid % 16;
-            double acc = 0.0;
-            for (int s2 = 0; s2 < kb; ++s2) acc = fma(Ta[ti][s2], Tb[tj][s2], acc);
-            const int i = r0 + ti, j = c0 + tj;
-            if (i < nb1 && j <= i) {
+            const int nel = nb1 * (nb1 + 1) / 2;
+            const int e0 = pieces ? bid * PIECE : 0, e1 = pieces ? min(nel, e0 + PIECE) : nel;
+            for (int e = e0 + tid; e < e1; e += NT) {
+                const int i = tri[e] >> 8, j = tri[e] & 0xff;
                 double* c = p.V + (long long)(d0 + i) * R + d0 + j;
-                *c = __ldcg(c) - acc;
+                const double c0 = __ldcg(c);
+                double acc = 0.0;
+#pragma unroll 8
+                for (int s2 = 0; s2 < NB; ++s2) acc = fma(Ta[i][s2], Ta[j][s2], acc);
+                if (bid == 0)
+                    Ls[i][j] = c0 - acc;
+                else
+                    *c = c0 - acc;
             }
             __syncthreads();
-            if (q > 0) {
+            if (bid != 0) {
                 if (tid == 0) atom_add_release(&p.sync[3], 1u);
             } else {
-                if (tid == 0) {
-                    int ok = 1;
-                    const unsigned int target = 2u * (unsigned int)(k + 1);
-                    const unsigned long long t0 = gtimer();
-                    while (ld_acquire(&p.sync[3]) < target) {
-                        if (ld_vol(&p.sync[2])) {
-                            ok = 0;
-                            break;
-                        }
-                        if (gtimer() - t0 > p.wait_ns) {
-                            atomicExch(&p.sync[2], 1u);
-                            atomicOr(p.err, 64u);
-                            ok = 0;
-                            break;
-                        }
+                if (pieces) {
+                    if (tid == 0)
+                        s_flag = poll_until(p, &p.sync[3], (unsigned int)(NPIECE - 1) * (unsigned int)(k + 1), 64u) ? 1 : 0;
+                    __syncthreads();
+                    for (int e = PIECE + tid; e < nel; e += NT) {
+                        const int i = tri[e] >> 8, j = tri[e] & 0xff;
+                        Ls[i][j] = __ldcg(p.V + (long long)(d0 + i) * R + d0 + j);
                     }
-                    s_flag = ok;
+                    __syncthreads();
                 }
-                __syncthreads();
-                if (s_flag) factor_block(p, k + 1, tol, Ls, Li, rd, tri, Tb);
+                if (!pieces || s_flag) factor_block(p.Linv + (long long)(k + 1) * NB * NB, nb1, tol, p.nclamp);
             }
         }
-        int first, stride;
-        if (G == 1) {
-            first = 0;
-            stride = 1;
-        } else if (bid == 0) {
-            first = split0 ? ntile : 0;   // tile 0 only, unless split above
-            stride = ntile + 1;
-        } else {
-            first = bid;
-            stride = G - 1;
-        }
+        // tiles 1 .. of the others (tile 0 is done above whenever there is one)
+        const int first = G == 1 ? 1 : (bid == 0 ? ntile : bid), stride = G == 1 ? 1 : G - 1;
         // each block's tiles in turn; the operands and the C values of the next
         // tile are loaded into registers while the current one is multiplied
         TrailTile cur{}, nxt{};
@@ -643,10 +655,9 @@ __device__ __forceinline__ void solve_body(const SolveP& p, const int bid, const
                 if (trail_owns(cur, i, j)) cur.C[(long long)i * R + j] = c4[u] - acc[u];
             }
             __syncthreads();
-            if (tile == 0 && k + 1 < nt && !split0) factor_block(p, k + 1, tol, Ls, Li, rd, tri, Tb);
             cur = nxt;
         }
-        if (!gsync(p, gen, &s_flag, bid, G)) return;
+        if (!gsync(p, target, &s_flag, bid, G)) return;
     }
 
     // ---- P2: back substitution U~ L = Z, RB rows at a time ------------------------
@@ -656,16 +667,16 @@ __device__ __forceinline__ void solve_body(const SolveP& p, const int bid, const
         const int rbeg = bid * rpc, rend = min(dim, rbeg + rpc);
         for (int r0 = rbeg; r0 < rend; r0 += RB) {
             switch (min(RB, rend - r0)) {
-                case 4: back_rows<4>(p, r0, xs, Ls, Li); break;
-                case 3: back_rows<3>(p, r0, xs, Ls, Li); break;
-                case 2: back_rows<2>(p, r0, xs, Ls, Li); break;
-                default: back_rows<1>(p, r0, xs, Ls, Li); break;
+                case 4: back_rows<4>(p, r0, xs, Ls, Li, Ta, Tb); break;
+                case 3: back_rows<3>(p, r0, xs, Ls, Li, Ta, Tb); break;
+                case 2: back_rows<2>(p, r0, xs, Ls, Li, Ta, Tb); break;
+                default: back_rows<1>(p, r0, xs, Ls, Li, Ta, Tb); break;
             }
         }
     }
     constexpr int T16 = 16;
     const int ty16 = tid / T16, tx16 = tid % T16;
-    if (!gsync(p, gen, &s_flag, bid, G)) return;
+    if (!gsync(p, target, &s_flag, bid, G)) return;
 
     // ---- P3: normalise: 32 columns per block, 8 row groups, a zero column keeps lam = 0
     {
@@ -695,7 +706,7 @@ __device__ __forceinline__ void solve_body(const SolveP& p, const int bid, const
             __syncthreads();
         }
     }
-    if (!gsync(p, gen, &s_flag, bid, G)) return;
+    if (!gsync(p, target, &s_flag, bid, G)) return;
 
     // ---- P4: Gram of the new factor, 16 x 16 tiles of the lower triangle ------------
     const int TR = (R + T16 - 1) / T16;
@@ -755,7 +766,10 @@ __device__ __forceinline__ void solve_body(const SolveP& p, const int bid, const
     }
 }
 
-__global__ void __launch_bounds__(NT, 1) k_solve(const __grid_constant__ SolveP p) { solve_body(p, blockIdx.x, gridDim.x); }
+__global__ void __launch_bounds__(NT, 1) k_solve(const __grid_constant__ SolveP p) {
+    solve_body(p, blockIdx.x, gridDim.x);
+    leave_sync(p, gridDim.x);
+}
 
 // Several instances' mode updates in one cooperative launch.  The blocks form
 // lanes: lane l is blocks lane_blk0[l] .. lane_blk0[l+1]-1 and solves the
@@ -777,16 +791,8 @@ __global__ void __launch_bounds__(NT, 3) k_solve_batch(const __grid_constant__ S
     const int bid = (int)blockIdx.x - b.lane_blk0[l], G = b.lane_blk0[l + 1] - b.lane_blk0[l];
     for (int i = b.lane_inst0[l]; i < b.lane_inst0[l + 1]; ++i) {
         solve_body(b.p[b.order[i]], bid, G);
+        leave_sync(b.p[b.order[i]], G);
         __syncthreads();   // the block's shared memory is reused by the next instance
-    }
-}
-
-// the barrier words and the diagonal maximum of every instance start at zero
-__global__ void k_solve_batch_prep(const __grid_constant__ SolveBatch b) {
-    const int k = threadIdx.x;
-    if (k < b.n) {
-        for (int w = 0; w < 4; ++w) b.p[k].sync[w] = 0u;
-        *b.p[k].maxdiag = 0ull;
     }
 }
 
@@ -800,7 +806,7 @@ SolveP to_params(const SolveArgs& a) {
     SolveP p;
     p.G1 = a.G1; p.G2 = a.G2; p.G3 = a.G3; p.V = a.V; p.Linv = a.Linv; p.M = a.M; p.Z = a.Z;
     p.U = a.U; p.lam = a.lam; p.G = a.G;
-    p.sync = a.sync; p.maxdiag = a.maxdiag; p.nclamp = a.nclamp; p.err = a.err; p.R = a.R; p.dim = a.dim;
+    p.sync = a.sync; p.nclamp = a.nclamp; p.err = a.err; p.R = a.R; p.dim = a.dim;
     p.withhold = a.withhold;
     p.wait_ns = a.wait_ns > 0 ? a.wait_ns : BAR_NS;
     return p;
@@ -835,16 +841,14 @@ int g_batch_per_sm = 0;
 
 int solve_mode_coop(const double* G1, const double* G2, const double* G3, const double* M, int dim, int R,
                     double* V, double* Linv, double* Z, double* U, double* lam, double* G,
-                    unsigned int* sync, unsigned long long* maxdiag, unsigned long long* nclamp, unsigned int* err,
+                    unsigned int* sync, unsigned long long* nclamp, unsigned int* err,
                     int grid_cap, unsigned long long wait_ns, unsigned int* withhold, cudaStream_t s) {
     const int sms = sm_total();
     if (sms <= 0) return -1;
     // small problems take fewer blocks, so that several instances' solves can share the GPU
     int grid = solve_want(dim, R, sms);
     if (grid_cap > 0 && grid > grid_cap) grid = grid_cap < 8 ? 8 : grid_cap;
-    cudaMemsetAsync(sync, 0, 4 * sizeof(unsigned int), s);
-    cudaMemsetAsync(maxdiag, 0, sizeof(unsigned long long), s);
-    SolveArgs a{G1, G2, G3, M, dim, R, V, Linv, Z, U, lam, G, sync, maxdiag, nclamp, err, wait_ns, withhold};
+    SolveArgs a{G1, G2, G3, M, dim, R, V, Linv, Z, U, lam, G, sync, nclamp, err, wait_ns, withhold};
     const SolveP p = to_params(a);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
@@ -933,7 +937,6 @@ int solve_modes_batched(const SolveArgs* a, int n, cudaStream_t s) {
         }
         b.lane_blk0[best_L] = blk;
         b.lane_inst0[best_L] = q;
-        k_solve_batch_prep<<<1, MAX_BATCH, 0, s>>>(b);
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(blk);
         cfg.blockDim = dim3(NT);

@@ -162,6 +162,28 @@ def test_fp64_sweeps_match_oracle(shape):
     cp.close()
 
 
+@pytest.mark.parametrize("R", [2, 31, 32, 33, 63, 64, 65, 161])
+def test_solve_at_block_edges(R):
+    """The solve's 32-wide blocks at their edges (a last block of 1, 2, 31 or 32
+    columns, one to six blocks): FP64 sweeps against the oracle, with the clamped
+    pivots counted alike (R = 161 exceeds the rank 10 * 4 * 4 of V for modes a and
+    b, so it is singular there and only the first sweep's count is compared)."""
+    o, v, X = 4, 10, 12
+    inp = inputs.make_inputs(o, v, X, R, seed=13)
+    cp = binding.CpAls(_dev(inp.B), _dev(inp.tau), inp.factors, precision="fp64")
+    if R == 161:
+        cp.sweep(1)
+        assert cp.stats()["clamped_pivots"] >= 1
+        f = _factors(cp)
+        assert all(np.all(np.isfinite(x)) for x in f.values())
+    else:
+        U_ref, lam_ref, hist = orc.cp_als(inp.Bvv, inp.tau, inp.factors, 2)
+        cp.sweep(2)
+        _check_factors(_factors(cp), U_ref, lam_ref, 1e-8, f"fp64 R={R} after 2 sweeps")
+        assert cp.stats()["clamped_pivots"] == sum(h["nclamped"] for h in hist)
+    cp.close()
+
+
 @pytest.mark.parametrize("shape", SHAPES[:3])
 def test_exact_contraction_and_energies(shape):
     o, v, X, R = shape
