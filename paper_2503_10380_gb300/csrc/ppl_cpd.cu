@@ -42,6 +42,8 @@ struct Layout {
     size_t Za, Zb, gov, Gblk, Rblk;
     size_t ring, cache, guess0;   // 6 iterates, the Near-Optimal cache, the initial guess
     size_t recon;                 // Khatri-Rao chunks for the reconstruction
+    size_t rowx;                  // eight bytes per operand row of an FP64 contraction
+    long long nrowx;
     int rcr;
     size_t total;
     int rc, na;
@@ -65,6 +67,7 @@ constexpr int RC_MAX = 1024; // most rank columns per pass of the chain
 #ifndef BATCH_SOLVE_SHARE
 #define BATCH_SOLVE_SHARE 4     // a batched solve takes about SHARE / nstreams of the SMs
 #endif
+constexpr int FP64_KSPLIT = 608; // most split-K slices of an FP64 contraction
 constexpr int NSCAL = 64;
 // scalar slots
 constexpr int SC_TERMS = 2, SC_NORMR2 = 8, SC_NORM2_PREV = 9, SC_CROSS = 10, SC_ENERGY = 12,
@@ -138,8 +141,20 @@ bool plan(int o, int v, int X, int R, const ppl_cpd_opts& op, Layout& L) {
     L.ring = take(6 * fsz);
     L.cache = take(fsz);
     L.guess0 = take(fsz);
-    L.rcr = R < 64 ? R : 64;
+    L.rcr = R < 256 ? R : 256;
     L.recon = take((size_t)((long long)v * v + (long long)o * o) * L.rcr * d);
+    // the widest pair of operands: W or the dressing (X v and rc or v rows), Y or S (per
+    // batch entry), the energy, the exact contraction, the reconstruction, a Gram matrix
+    {
+        const long long xv = (long long)X * v, vv = (long long)v * v, oo = (long long)o * o;
+        const long long pairs[] = {xv + v + rc, (long long)rc * ((long long)X + 2 * v), (long long)X * o + R, vv + oo + R,
+                                   na * v + vv + oo, 2ll * o * v, 2ll * R,
+                                   // split over K: M and P of the FP64 form, up to FP64_KSPLIT slices
+                                   (long long)FP64_KSPLIT * (v + rc), (long long)FP64_KSPLIT * (oo + rc)};
+        L.nrowx = 0;
+        for (long long n : pairs) L.nrowx = n > L.nrowx ? n : L.nrowx;
+        L.rowx = take((size_t)L.nrowx * sizeof(unsigned long long));
+    }
     const size_t none = (size_t)-1;
     L.T64 = L.W64 = L.Y64 = L.S64 = none;
     L.tauT = L.tauN = L.Bn = L.Bp = L.BpW = L.UopA = L.UopB = L.KRT = L.T = L.Tt = L.W = L.Y = L.WTa = L.WTb = L.S = none;
@@ -404,6 +419,13 @@ int run_tc(ppl_cpd* h, TcGemm& g, const char* what) {
 
 // ---- FP64 pieces shared by both precisions ------------------------------------
 
+void gemm(ppl_cpd* h, G64& g) {
+    g.err = h->errflag();
+    g.scratch = h->at<unsigned long long>(h->L.rowx);
+    g.nscratch = h->L.nrowx;
+    gemm64(g, h->st);
+}
+
 void gram(ppl_cpd* h, int m) {
     G64 g{};
     const int R = h->R;
@@ -411,7 +433,7 @@ void gram(ppl_cpd* h, int m) {
     g.B = h->U[m]; g.bn = ix1(1); g.bk = ix1(R);
     g.C = h->G(m); g.cm = ix1(R); g.cn = ix1(1);
     g.M = R; g.N = R; g.K = h->dim(m); g.batch = 1; g.ksplit = 1; g.alpha = 1.0;
-    gemm64(g, h->st);
+    gemm(h, g);
 }
 
 // the arguments of mode m's update: V from the other three Gram matrices, M from L.M
@@ -454,7 +476,7 @@ void t_fp64(ppl_cpd* h) {
     g.B = h->tau; g.bn = ix1(1); g.bk = ix1((long long)v * v);
     g.C = h->at<double>(h->L.T64); g.cm = ix1((long long)v * v); g.cn = ix1(1);
     g.M = R; g.N = v * v; g.K = o * o; g.batch = 1; g.ksplit = 1; g.alpha = 1.0;
-    gemm64(g, h->st);
+    gemm(h, g);
 }
 
 // W[r][Q][d] = sum_b B[Q][o+b][o+d] U[b][r0+r]; bside: the dressed D-bar[Q][b][d]
@@ -469,7 +491,7 @@ void w_fp64(ppl_cpd* h, const double* U, int r0, int rcur, double* W, bool bside
     g.B = U + r0; g.bn = ix1(1); g.bk = ix1(R);
     g.C = W; g.cm = ix1(1); g.cn = ix1((long long)X * v);
     g.M = X * v; g.N = rcur; g.K = v; g.batch = 1; g.ksplit = 1; g.alpha = 1.0;
-    gemm64(g, h->st);
+    gemm(h, g);
 }
 
 void mttkrp_ab_fp64(ppl_cpd* h, int mode, double* Mout) {
@@ -488,7 +510,7 @@ void mttkrp_ab_fp64(ppl_cpd* h, int mode, double* Mout) {
         else           { y.bn = ix1(1); y.bk = ix1(v); }   // T[r][c][d], contract c
         y.C = Y; y.cb = (long long)X * v; y.cm = ix1(v); y.cn = ix1(1);
         y.M = X; y.N = v; y.K = v; y.batch = rcur; y.ksplit = 1; y.alpha = 1.0;
-        gemm64(y, h->st);
+        gemm(h, y);
         G64 m{};
         if (mode == 1 && h->dressed()) {
             m.A = h->at<double>(h->L.Bbar); m.am = ix1(v); m.ak = ix2(v, (long long)v * v, 1);
@@ -499,10 +521,10 @@ void mttkrp_ab_fp64(ppl_cpd* h, int mode, double* Mout) {
         m.C = Mout + r0; m.cm = ix1(R); m.cn = ix1(1);
         m.M = v; m.N = rcur; m.K = X * v; m.batch = 1; m.alpha = 1.0; m.atomic = 1;
         const long long tiles = (long long)((v + 63) / 64) * ((rcur + 63) / 64);
-        long long ks = (608 + tiles - 1) / tiles;
+        long long ks = (FP64_KSPLIT + tiles - 1) / tiles;
         if (ks > (X * (long long)v) / 64) ks = (X * (long long)v) / 64;
         m.ksplit = ks < 1 ? 1 : (int)ks;
-        gemm64(m, h->st);
+        gemm(h, m);
     }
 }
 
@@ -522,17 +544,17 @@ void p_fp64(ppl_cpd* h) {
         s.B = Wb; s.bb = (long long)X * v; s.bn = ix1(1); s.bk = ix1(v);
         s.C = S; s.cb = (long long)v * v; s.cm = ix1(v); s.cn = ix1(1);
         s.M = v; s.N = v; s.K = X; s.batch = rcur; s.ksplit = 1; s.alpha = 1.0;
-        gemm64(s, h->st);
+        gemm(h, s);
         G64 p{};
         p.A = h->tau; p.am = ix1((long long)v * v); p.ak = ix1(1);
         p.B = S; p.bn = ix1((long long)v * v); p.bk = ix1(1);
         p.C = P + r0; p.cm = ix1(R); p.cn = ix1(1);
         p.M = o * o; p.N = rcur; p.K = v * v; p.batch = 1; p.alpha = 1.0; p.atomic = 1;
         const long long tiles = (long long)((o * o + 63) / 64) * ((rcur + 63) / 64);
-        long long ks = (608 + tiles - 1) / tiles;
+        long long ks = (FP64_KSPLIT + tiles - 1) / tiles;
         if (ks > (long long)v * v / 64) ks = (long long)v * v / 64;
         p.ksplit = ks < 1 ? 1 : (int)ks;
-        gemm64(p, h->st);
+        gemm(h, p);
     }
 }
 
@@ -775,7 +797,7 @@ void build_dbar(ppl_cpd* h, const double* t1) {
         g.B = t1; g.bn = ix1(1); g.bk = ix1(v);                                            // t1[k][d]
         g.C = Bb; g.cb = (long long)v * v; g.cm = ix1(v); g.cn = ix1(1);
         g.M = v; g.N = v; g.K = o; g.batch = X; g.ksplit = 1; g.alpha = -2.0; g.beta = 1.0;
-        gemm64(g, h->st);
+        gemm(h, g);
     }
     if (!h->tc()) return;
     // D-bar[Q][b][d] is not symmetric in (b, d): the b side of every contraction reads it with b as the row index
@@ -856,7 +878,7 @@ void cross_gram(ppl_cpd* h, int m) {
     g.B = h->at<double>(h->L.Uold[m]); g.bn = ix1(1); g.bk = ix1(R);
     g.C = h->at<double>(h->L.Xc[m]); g.cm = ix1(R); g.cn = ix1(1);
     g.M = R; g.N = R; g.K = h->dim(m); g.batch = 1; g.ksplit = 1; g.alpha = 1.0;
-    gemm64(g, h->st);
+    gemm(h, g);
 }
 
 // phase boundary; External makes the record a real event node when the
@@ -1209,11 +1231,12 @@ int ppl_cpd_energy(ppl_cpd* h, double* E_cp) {
     double* Z[2] = {h->at<double>(h->L.Za), h->at<double>(h->L.Zb)};
     for (int w = 0; w < 2; ++w) {
         G64 g{};
-        g.A = h->B + o; g.ab = (long long)n * n; g.am = ix1(n); g.ak = ix1(1);
+        // (Q, i) as one row index: o alone is far from filling a tile's rows
+        g.A = h->B + o; g.am = ix2(o, (long long)n * n, n); g.ak = ix1(1);
         g.B = h->U[w]; g.bn = ix1(1); g.bk = ix1(R);
-        g.C = Z[w]; g.cb = (long long)o * R; g.cm = ix1(R); g.cn = ix1(1);
-        g.M = o; g.N = R; g.K = v; g.batch = X; g.ksplit = 1; g.alpha = 1.0;
-        gemm64(g, h->st);
+        g.C = Z[w]; g.cm = ix1(R); g.cn = ix1(1);
+        g.M = X * o; g.N = R; g.K = v; g.batch = 1; g.ksplit = 1; g.alpha = 1.0;
+        gemm(h, g);
     }
     energy_reduce(Z[0], Z[1], h->U[2], h->U[3], h->lam, X, o, R, h->at<double>(h->L.partial),
                   h->scal() + SC_ENERGY, h->st);
@@ -1240,7 +1263,7 @@ int ppl_exact_contract(ppl_cpd* h, double* normR2, double* E_exact, double* R_ou
     g.B = h->B + o; g.bn = ix2(v, n, 1); g.bk = ix1((long long)n * n);
     g.C = gov; g.cm = ix1((long long)o * v); g.cn = ix1(1);
     g.M = o * v; g.N = o * v; g.K = X; g.batch = 1; g.ksplit = 1; g.alpha = 1.0;
-    gemm64(g, h->st);
+    gemm(h, g);
     const long long v3 = (long long)v * v * v, vo2 = (long long)v * o * o;
     for (int a0 = 0; a0 < v; a0 += na) {
         const int nb = (v - a0 < na) ? v - a0 : na;
@@ -1254,7 +1277,7 @@ int ppl_exact_contract(ppl_cpd* h, double* normR2, double* E_exact, double* R_ou
         }
         q.C = Gb; q.cb = v3; q.cm = ix1((long long)v * v); q.cn = ix1(1);
         q.M = v; q.N = v * v; q.K = X; q.batch = nb; q.ksplit = 1; q.alpha = 1.0;
-        gemm64(q, h->st);
+        gemm(h, q);
         // R[a][b][ij] = sum_{c,d} G_a[c][b][d] tau[ij][c][d]
         double* Rdst = R_out ? R_out + (long long)a0 * vo2 : Rb;
         G64 r{};
@@ -1262,7 +1285,7 @@ int ppl_exact_contract(ppl_cpd* h, double* normR2, double* E_exact, double* R_ou
         r.B = h->tau; r.bb = 0; r.bn = ix1((long long)v * v); r.bk = ix1(1);
         r.C = Rdst; r.cb = vo2; r.cm = ix1((long long)o * o); r.cn = ix1(1);
         r.M = v; r.N = o * o; r.K = v * v; r.batch = nb; r.ksplit = 1; r.alpha = 1.0;
-        gemm64(r, h->st);
+        gemm(h, r);
         exact_reduce(Rdst, a0, nb, v, o, gov, h->at<double>(h->L.partial), acc, h->st);
     }
     e = check_cuda(h, "exact_contract");
@@ -1294,7 +1317,7 @@ int ppl_cpd_reconstruct(ppl_cpd* h, double* R_out, int symmetrise) {
         g.C = R_out; g.cm = ix1((long long)o * o); g.cn = ix1(1);
         g.M = v * v; g.N = o * o; g.K = rc; g.batch = 1; g.ksplit = 1;
         g.alpha = 1.0; g.beta = (r0 == 0) ? 0.0 : 1.0;
-        gemm64(g, h->st);
+        gemm(h, g);
     }
     if (symmetrise) symmetrise_pairs(R_out, v, o, h->st);
     e = check_cuda(h, "reconstruct");
@@ -1318,7 +1341,7 @@ int ppl_exact_contract_mixed(ppl_cpd* h, double* normR2, double* E_exact, double
     g.B = h->B + o; g.bn = ix2(v, n, 1); g.bk = ix1((long long)n * n);
     g.C = gov; g.cm = ix1((long long)o * v); g.cn = ix1(1);
     g.M = o * v; g.N = o * v; g.K = X; g.batch = 1; g.ksplit = 1; g.alpha = 1.0;
-    gemm64(g, h->st);
+    gemm(h, g);
     const Pan pq = pan_of(h);
     const long long pQ = (long long)v * v * pq.kX, pG = (long long)v * pq.kvv;
     for (int a = 0; a < v && !e; ++a) {

@@ -2,6 +2,7 @@
 // form, and the Gram / Hadamard / Cholesky / triangular-solve / normalise /
 // fit / energy steps that run in FP64 in every precision mode.
 #include "ppl_internal.h"
+#include "ppl_gemm64.cuh"
 
 #include "../../include/ppl_cpd.h"
 
@@ -10,95 +11,16 @@
 
 namespace {
 
-constexpr int GBM = 64, GBN = 64, GBK = 16;
-
-__device__ __forceinline__ long long ixd(const Idx2& x, int i) {
-    return (long long)(i / x.div) * x.hi + (long long)(i % x.div) * x.lo;
-}
-
-// 64x64 output tile per CTA, 256 threads, 4x4 outputs per thread at
-// (ty + 16 i, tx + 16 j).  Operands are read through Idx2 maps, so every
-// layout of the method is served without copies; the FP64 pipe (not the
-// loads) bounds this kernel on GB300.
-__global__ void __launch_bounds__(256) k_gemm64(G64 g) {
+// One 64 x 64 output tile per block.
+__global__ void __launch_bounds__(256) k_gemm64(const __grid_constant__ G64 g) {
     const int b = blockIdx.z / g.ksplit, ks = blockIdx.z % g.ksplit;
     const int m0 = blockIdx.x * GBM, n0 = blockIdx.y * GBN;
     if (g.lower && n0 > m0 + GBM - 1) return;
     const int per = (((g.K + g.ksplit - 1) / g.ksplit) + GBK - 1) / GBK * GBK;
     const int kbeg = ks * per, kend = min(g.K, kbeg + per);
     if (kbeg >= kend && g.atomic) return;
-
-    __shared__ double As[GBK][GBM];
-    __shared__ double Bs[GBK][GBN];
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    const double* A = g.A + (long long)b * g.ab;
-    const double* B = g.B + (long long)b * g.bb;
-    const bool a_kfast = (g.ak.lo == 1 && g.ak.div >= (1 << 30));
-    const bool b_kfast = (g.bk.lo == 1 && g.bk.div >= (1 << 30));
-
-    // per-thread load coordinates: 4 elements of each 64x16 tile
-    int a_ml[4], a_kl[4], b_nl[4], b_kl[4];
-    long long a_row[4], b_row[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int e = tid + 256 * q;
-        a_ml[q] = a_kfast ? e / GBK : e % GBM;
-        a_kl[q] = a_kfast ? e % GBK : e / GBM;
-        b_nl[q] = b_kfast ? e / GBK : e % GBN;
-        b_kl[q] = b_kfast ? e % GBK : e / GBN;
-        const int m = m0 + a_ml[q], n = n0 + b_nl[q];
-        a_row[q] = (m < g.M) ? ixd(g.am, m) : -1;
-        b_row[q] = (n < g.N) ? ixd(g.bn, n) : -1;
-    }
-
-    double acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-
-    for (int k0 = kbeg; k0 < kend; k0 += GBK) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int ka = k0 + a_kl[q], kb = k0 + b_kl[q];
-            As[a_kl[q]][a_ml[q]] = (a_row[q] >= 0 && ka < kend) ? A[a_row[q] + ixd(g.ak, ka)] : 0.0;
-            Bs[b_kl[q]][b_nl[q]] = (b_row[q] >= 0 && kb < kend) ? B[b_row[q] + ixd(g.bk, kb)] : 0.0;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < GBK; ++kk) {
-            double av[4], bv[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) av[i] = As[kk][ty + 16 * i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) bv[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-
-    double* C = g.C + (long long)b * g.cb;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int m = m0 + ty + 16 * i;
-        if (m >= g.M) continue;
-        const long long cr = ixd(g.cm, m);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int n = n0 + tx + 16 * j;
-            if (n >= g.N) continue;
-            double* p = C + cr + ixd(g.cn, n);
-            if (g.atomic) {
-                atomicAdd(p, g.alpha * acc[i][j]);
-            } else {
-                const double old = (g.beta != 0.0) ? g.beta * *p : 0.0;
-                *p = fma(g.alpha, acc[i][j], old);
-            }
-        }
-    }
+    __shared__ double sm[GBK * (GBM + GBN)];
+    gemm64_tile(g, b, m0, n0, kbeg, kend, sm);
 }
 
 __global__ void k_kr(const double* Ui, const double* Uj, int o, int R, double* KR, int ld) {
@@ -352,6 +274,8 @@ void gemm64(const G64& g, cudaStream_t s) {
         }
         return;
     }
+    // On the tensor cores where the caller gives an error word for its bounded waits.
+    if (g.err && g.K >= SPLIT64_MIN_K && gemm64_split(g, s) == 0) return;
     k_gemm64<<<grid, 256, 0, s>>>(g);
 }
 

@@ -24,8 +24,19 @@ struct G64 {
     double alpha, beta;
     int atomic;   // 1: atomicAdd(alpha * acc) into C (split-K); beta ignored
     int lower;    // 1: skip tiles whose columns all lie above the diagonal (n > m)
+    // for the tensor cores (nullptr: CUDA cores only): the error word of bounded device
+    // waits, and room for eight bytes per row of A and B (per split-K slice, and per
+    // batch entry where ab, bb != 0)
+    unsigned int* err;
+    unsigned long long* scratch;
+    long long nscratch;
 };
 void gemm64(const G64& g, cudaStream_t s);
+// the same on the tensor cores by exact digit products (ppl_split64.cu), with g.err and
+// g.scratch; nonzero (nothing launched) where the shape is out of its range
+int gemm64_split(const G64& g, cudaStream_t s);
+// from this K on: a k block of 32 costs 8k clocks however few are used, the CUDA cores 2k per k and tile
+constexpr int SPLIT64_MIN_K = 8;
 
 // ---- small FP64 kernels (ppl_fp64.cu) -------------------------------------
 // KR[r][i*o+j] = Ui[i][r] * Uj[j][r]   (FP64, [R][ld])

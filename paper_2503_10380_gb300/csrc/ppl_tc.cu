@@ -25,6 +25,7 @@
 // Every mbarrier wait is bounded; on expiry the kernel records the error,
 // drains what it issued, frees TMEM and returns.
 #include "ppl_internal.h"
+#include "ppl_ptx.cuh"
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -109,46 +110,6 @@ template <int PREC> struct Prec {
     static constexpr int KSTEP = HALF ? 16 : 8;                // K per MMA instruction
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ unsigned long long gtimer() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t a, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(a), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t a, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(a), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try(uint32_t a, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(a), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// bounded wait: true when the phase completed, false after limit_ns
-__device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, unsigned long long limit_ns) {
-    if (mbar_try(a, parity)) return true;
-    const unsigned long long t0 = gtimer();
-    while (true) {
-        if (mbar_try(a, parity)) return true;
-        if (gtimer() - t0 > limit_ns) return false;
-    }
-}
-
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2,
                                             uint32_t mbar) {
     asm volatile(
@@ -176,17 +137,6 @@ __device__ __forceinline__ void load_op(uint32_t dst, const CUtensorMap* map, bo
         tma_load_3d(dst, map, kb * ke, row, b, mbar);
 }
 
-// shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 B apart
-__device__ __forceinline__ unsigned long long make_desc(uint32_t saddr) {
-    unsigned long long d = 0;
-    d |= (unsigned long long)((saddr & 0x3FFFFu) >> 4);
-    d |= 1ull << 16;                       // leading byte offset (unused for swizzled K-major)
-    d |= (unsigned long long)(1024 >> 4) << 32;   // stride byte offset
-    d |= 1ull << 46;                       // descriptor version
-    d |= 2ull << 61;                       // SWIZZLE_128B
-    return d;
-}
-
 template <int PREC>
 __device__ __forceinline__ void mma(uint32_t tmem, unsigned long long ad, unsigned long long bd, uint32_t idesc,
                                     uint32_t acc) {
@@ -203,11 +153,6 @@ __device__ __forceinline__ void mma(uint32_t tmem, unsigned long long ad, unsign
             "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
             : "memory");
     }
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t mbar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
-                 : "memory");
 }
 
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {

@@ -378,6 +378,51 @@ def test_reconstruct_and_symmetrise(prec):
     cp.close()
 
 
+@pytest.mark.parametrize("o,v,R", [(1, 3, 8), (3, 11, 9), (8, 16, 31), (5, 12, 33), (9, 23, 130), (12, 33, 300)])
+@pytest.mark.parametrize("scale", ["even", "wide"])
+def test_fp64_contraction_by_digits(o, v, R, scale):
+    """The FP64 contraction formed from exact digit products: R~ (M = v^2, N = o^2,
+    K = the rank columns) at ragged tiles and k blocks, element by element within
+    the bound of the FP64 sums.  "wide": column r of U_a scaled by 10^s and of U_i by
+    10^-s, s up to 12, so that the entries a row is scaled by meet the other
+    operand's smallest ones and the fixed-point digits alone would be 1e-5 off."""
+    inp = inputs.make_inputs(o, v, 2 * v, R, seed=14)
+    f = {m: x.copy() for m, x in inp.factors.items()}
+    if scale == "wide":
+        s = np.random.default_rng(1).uniform(-12, 12, R)
+        f["a"] *= 10.0 ** s
+        f["i"] *= 10.0 ** -s
+    cp = binding.CpAls(_dev(inp.B), _dev(inp.tau), f, precision="fp64")
+    ref = orc.reconstruct(f, np.ones(R))
+    ref_abs = orc.reconstruct(abs_factors(f), np.ones(R))
+    check_abs_bound(cp.reconstruct(False).cpu().numpy(), ref, ref_abs, 1e-13, f"{scale} {(o, v, R)}")
+    cp.close()
+
+
+@pytest.mark.parametrize("what", ["inf", "nan", "denormal", "zero"])
+def test_fp64_contraction_special_values(what):
+    """An Inf, a NaN, a row of denormals or a zero row in a factor: the same
+    elements of R~ are infinite, NaN or zero as in an FP64 sum, the others are as
+    accurate as before."""
+    o, v, R = 6, 13, 40
+    inp = inputs.make_inputs(o, v, 2 * v, R, seed=15)
+    f = {m: x.copy() for m, x in inp.factors.items()}
+    x = {"inf": np.inf, "nan": np.nan, "denormal": 3e-310, "zero": 0.0}[what]
+    if what in ("inf", "nan"):
+        f["b"][4, 17] = x
+    else:
+        f["b"][4, :] = x
+    cp = binding.CpAls(_dev(inp.B), _dev(inp.tau), f, precision="fp64")
+    got = cp.reconstruct(False).cpu().numpy()
+    with np.errstate(all="ignore"):
+        ref = np.einsum("ar,br,ir,jr->abij", f["a"], f["b"], f["i"], f["j"])
+        ref_abs = np.einsum("ar,br,ir,jr->abij", *(np.abs(f[m]) for m in "abij"))
+    assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(np.isinf(got), np.isinf(ref))
+    ok = np.isfinite(ref)
+    assert np.all(np.abs(got[ok] - ref[ok]) <= 1e-13 * ref_abs[ok] + 1e-320)
+    cp.close()
+
+
 def test_batch_of_uneven_instances_equals_individual_sweeps():
     shapes = [(4, 40, 120, 96), (6, 56, 168, 130), (5, 24, 72, 48), (8, 64, 192, 200)]
     probs, solo = [], []
