@@ -419,7 +419,16 @@ int run_tc(ppl_cpd* h, TcGemm& g, const char* what) {
 
 // ---- FP64 pieces shared by both precisions ------------------------------------
 
-void gemm(ppl_cpd* h, G64& g) {
+// An FP64 contraction.  `operand`: its result is split into tensor-core operands (the
+// Gram matrices of a guess through the solve, the dressed D-bar).  There the last bit
+// matters: at a rounding boundary of an operand it moves every later sweep by the
+// split precision's noise, so the tensor-core forms sum those on the CUDA cores, in
+// the order of k; nothing else does.
+void gemm(ppl_cpd* h, G64& g, bool operand = false) {
+    if (operand && h->tc()) {
+        gemm64(g, h->st);
+        return;
+    }
     g.err = h->errflag();
     g.scratch = h->at<unsigned long long>(h->L.rowx);
     g.nscratch = h->L.nrowx;
@@ -433,7 +442,8 @@ void gram(ppl_cpd* h, int m) {
     g.B = h->U[m]; g.bn = ix1(1); g.bk = ix1(R);
     g.C = h->G(m); g.cm = ix1(R); g.cn = ix1(1);
     g.M = R; g.N = R; g.K = h->dim(m); g.batch = 1; g.ksplit = 1; g.alpha = 1.0;
-    gemm(h, g);
+    g.lower = h->tc();     // symmetric: half the FP64 work
+    gemm(h, g, true);
 }
 
 // the arguments of mode m's update: V from the other three Gram matrices, M from L.M
@@ -797,7 +807,7 @@ void build_dbar(ppl_cpd* h, const double* t1) {
         g.B = t1; g.bn = ix1(1); g.bk = ix1(v);                                            // t1[k][d]
         g.C = Bb; g.cb = (long long)v * v; g.cm = ix1(v); g.cn = ix1(1);
         g.M = v; g.N = v; g.K = o; g.batch = X; g.ksplit = 1; g.alpha = -2.0; g.beta = 1.0;
-        gemm(h, g);
+        gemm(h, g, true);
     }
     if (!h->tc()) return;
     // D-bar[Q][b][d] is not symmetric in (b, d): the b side of every contraction reads it with b as the row index

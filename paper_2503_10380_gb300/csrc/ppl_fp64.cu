@@ -15,7 +15,7 @@ namespace {
 __global__ void __launch_bounds__(256) k_gemm64(const __grid_constant__ G64 g) {
     const int b = blockIdx.z / g.ksplit, ks = blockIdx.z % g.ksplit;
     const int m0 = blockIdx.x * GBM, n0 = blockIdx.y * GBN;
-    if (g.lower && n0 > m0 + GBM - 1) return;
+    if (g.lower && n0 > m0) return;
     const int per = (((g.K + g.ksplit - 1) / g.ksplit) + GBK - 1) / GBK * GBK;
     const int kbeg = ks * per, kend = min(g.K, kbeg + per);
     if (kbeg >= kend && g.atomic) return;

@@ -89,6 +89,7 @@ __device__ __forceinline__ void gemm64_tile(const G64& g, int b, int m0, int n0,
                 const double old = (g.beta != 0.0) ? g.beta * *p : 0.0;
                 *p = fma(g.alpha, acc[i][j], old);
             }
+            if (g.lower && n0 < m0) C[ixd(g.cm, n) + ixd(g.cn, m)] = *p;     // the mirrored tile
         }
     }
 }

@@ -23,7 +23,7 @@ struct G64 {
     int M, N, K, batch, ksplit;
     double alpha, beta;
     int atomic;   // 1: atomicAdd(alpha * acc) into C (split-K); beta ignored
-    int lower;    // 1: skip tiles whose columns all lie above the diagonal (n > m)
+    int lower;    // 1: C is symmetric: tiles right of the diagonal are copied from the left ones (no atomic, beta = 0)
     // for the tensor cores (nullptr: CUDA cores only): the error word of bounded device
     // waits, and room for eight bytes per row of A and B (per split-K slice, and per
     // batch entry where ab, bb != 0)

@@ -38,6 +38,7 @@ __shared__ double Ls[NB][NB + 1];   // the diagonal block being factored; stagin
 __shared__ double Li[NB][NB + 1];   // its column-scaled factor; staging in the back substitution
 __shared__ double Ta[NB][NB + 1];   // tiles
 __shared__ double Tb[NB][NB + 1];
+__shared__ double rd[NB];           // 1 / L_jj
 __shared__ unsigned short tri[NB * (NB + 1) / 2];   // (row << 8) | col of the lower triangle, row-major
 
 struct SolveP {
@@ -168,17 +169,21 @@ __device__ __forceinline__ void tri_index(int t, int& I, int& J) {
     J = t - i * (i + 1) / 2;
 }
 
-// 1/d for a positive normal d: the PTX approximate reciprocal (relative error e
-// about 2^-20) with one third-order step x <- x (1 + e + e^2), e = 1 - d x, whose
-// error is e^3 (Householder's method of order two).  Three dependent FP64 FMAs:
-// an FP64 warp instruction takes 64 clocks on GB300, issue and latency alike, and
-// the pivots' reciprocals are the factorisation's critical path (two Newton steps
-// are four).
+// 1/d for a positive normal d: the PTX approximate reciprocal refined by two
+// Newton-Raphson steps x <- x + x (1 - d x), each squaring the relative error
+// (within an ulp or two of the correctly rounded quotient).  Four FP64 FMAs
+// instead of the longer IEEE division sequence on the factorisation's
+// critical path.  (One third-order step is three, 64 clocks less per pivot, but its
+// last bits differ; the tensor-core forms split the factors into operands, and a
+// last bit at a rounding boundary of an operand changes every later sweep by the
+// split precision's noise.)
 __device__ __forceinline__ double recip_nr(double d) {
     double x;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(d));
-    const double e = fma(-d, x, 1.0);
-    return fma(x, fma(e, e, e), x);
+    double e = fma(-d, x, 1.0);
+    x = fma(x, e, x);
+    e = fma(-d, x, 1.0);
+    return fma(x, e, x);
 }
 
 // Factor the kb x kb diagonal block held in Ls (lower) and leave in Li the
@@ -187,15 +192,15 @@ __device__ __forceinline__ double recip_nr(double d) {
 // not above tol are replaced by tol and counted.  Li is also written to Linv, where
 // the other blocks read it.  All NT threads.
 //
-// Right-looking on unscaled columns: with d_j the pivot and s_i = a_ij / d_j
-// (which is Li[i][j]), a_ic -= s_i a_cj.  An FP64 instruction occupies its SM
+// Right-looking on unscaled columns: with d_j the pivot and s_i = a_ij (1 / d_j),
+// a_ic -= s_i a_cj; the scalings by 1 / sqrt(d_j) follow at the end, all at once.  An FP64 instruction occupies its SM
 // sub-partition's pipe for 64 clocks however many lanes are active, so the work
 // is laid out by sub-partitions.  Warp 0 alone, on its own sub-partition, owns the
 // chain pivot -> reciprocal -> column -> next pivot: at step j it scales column j
 // (which it hands to the others), updates column j + 1 and inverts the next pivot,
-// five dependent FP64 instructions, while the six warps of the other three
+// six dependent FP64 instructions, while the six warps of the other three
 // sub-partitions apply column j to columns j + 2 ..; one block barrier per step.
-// The pivot test is an integer comparison (an FP64 one is a sixth instruction).
+// The pivot test is an integer comparison (an FP64 one is one more instruction).
 // Measured on one 32 x 32 block: 16.3 us with the whole triangle updated by all
 // warps, two instructions per element, the reciprocal after it in the same step
 // and separate passes for square roots and scaling; 10.5 us so.
@@ -251,7 +256,13 @@ __device__ __noinline__ void factor_block(double* Linv, int kb, double tol, unsi
         }
         __syncthreads();
     }
-    if (warp == 0 && lane < kb) Li[lane][lane] = rsqrt(dl);
+    // L_jj = sqrt(d_j), L_ij = a_ij / L_jj, Li_ij = L_ij / L_jj
+    if (warp == 0) rd[lane] = lane < kb ? recip_nr(sqrt(dl)) : 0.0;
+    __syncthreads();
+    for (int e = threadIdx.x; e < kb * (kb + 1) / 2; e += NT) {
+        const int i = tri[e] >> 8, j = tri[e] & 0xff;
+        Li[i][j] = i == j ? rd[i] : Ls[i][j] * rd[j] * rd[j];
+    }
     __syncthreads();
     for (int e = threadIdx.x; e < NB * NB; e += NT) Linv[e] = Li[e / NB][e % NB];
     __syncthreads();

@@ -315,7 +315,6 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
     const int t = blockIdx.x;
     const int mt = ntm <= ntn ? t % ntm : t / ntn, nt = ntm <= ntn ? t / ntm : t % ntn;
     const int m0 = mt * EM, n0 = nt * EN;
-    if (g.lower && n0 > m0 + EM - 1) return;
     const int b = blockIdx.z / g.ksplit, ks = blockIdx.z % g.ksplit;
     const int per = slice_len(g.K, g.ksplit);
     const int kbeg = ks * per, kend = min(g.K, kbeg + per);
@@ -633,6 +632,7 @@ int gemm64_split(const G64& g, cudaStream_t s) {
         if (fa.numRegs != EREG_LAUNCH || fa.maxThreadsPerBlock < ETHREADS) return -3;
         attr = true;
     }
+    if (g.lower) return -5;        // (Gram matrices of the CUDA-core form only)
     const long long tiles = (long long)((g.M + EM - 1) / EM) * ((g.N + EN - 1) / EN);
     const long long z = (long long)g.batch * g.ksplit;
     // grid limits, and K 2^38 of the integer sums below 2^63
