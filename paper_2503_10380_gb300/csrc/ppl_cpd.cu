@@ -336,8 +336,8 @@ Ix plain(long long s, int ke) { return Ix{ke * s, s}; }
 // the consumer's K index inside its K panels, panels pstride elements apart
 Ix kpan(long long pstride) { return Ix{pstride, 1}; }
 
-// EPI_SPLIT output: element (m, n) of batch b at b*sb + map(m / mdiv, m % mdiv) + map(n)
-TcOut out_map(void* p, long long plane, long long sb, int mdiv, Ix q1, Ix q0, Ix n) {
+// EPI_SPLIT output: element (m, n) of batch b at b*sb + map(m / mdiv, m % mdiv) + n*ns
+TcOut out_map(void* p, long long plane, long long sb, int mdiv, Ix q1, Ix q0, long long ns) {
     TcOut o{};
     o.kind = EPI_SPLIT;
     o.out = p;
@@ -346,8 +346,7 @@ TcOut out_map(void* p, long long plane, long long sb, int mdiv, Ix q1, Ix q0, Ix
     o.mdiv = mdiv;
     o.q1p = q1.p; o.q1s = q1.s;
     o.q0p = q0.p; o.q0s = q0.s;
-    o.np = n.p; o.ns = n.s;
-    o.alpha = 1.0f;
+    o.ns = ns;
     return o;
 }
 
@@ -623,7 +622,7 @@ int t_tc(ppl_cpd* h) {
     g.B = pmat(opb(h, h->L.KRT), pKRT, R, o * o, 1, R, 0);
     g.M = v * v; g.N = R; g.K = o * o; g.batch = 1; g.ksplit = 1;
     // T[r]: rows c, K d; m = c*v + d, n = r
-    g.out = out_map(opb(h, h->L.T), pT, 0, v, plain(q.ke, q.ke), kpan((long long)v * q.ke), plain(bT, q.ke));
+    g.out = out_map(opb(h, h->L.T), pT, 0, v, plain(q.ke, q.ke), kpan((long long)v * q.ke), bT);
     int rc = run_tc(h, g, "T");
     if (rc) return rc;
     // T transposed per r: Tt[r] rows d, K c.  (A second copy written by the T
@@ -650,8 +649,7 @@ int run_tc_partial(ppl_cpd* h, TcGemm& g, double* out, long long ldo, const char
     g.out.out = part;
     g.out.sk = (long long)g.M * g.N;
     g.out.q0p = ke; g.out.q0s = 1;
-    g.out.np = (long long)ke * g.M; g.out.ns = g.M;
-    g.out.alpha = 1.0f;
+    g.out.ns = g.M;
     int e = run_tc(h, g, what);
     if (e) return e;
     reduce_partials(part, ks, g.M, g.N, out, ldo, h->st);
@@ -678,7 +676,7 @@ int chain_tc(ppl_cpd* h, int mode, double* Mout, bool keep_wa) {
         g1.A = pmat(opb(h, (mode == 0 && h->dressed()) ? h->L.BbN : h->L.Bn), pBn, X * v, v, 1, (long long)X * v, 0);
         g1.B = pmat(opb(h, h->L.UopA), pU, R, v, 1, R, 0);
         g1.M = X * v; g1.N = rcur; g1.K = v; g1.batch = 1; g1.ksplit = 1; g1.b_row0 = r0; g1.nfast = 1;
-        g1.out = out_map(opb(h, h->L.W), pW, 0, v, plain(q.ke, q.ke), kpan((long long)X * q.ke), plain(bW, q.ke));
+        g1.out = out_map(opb(h, h->L.W), pW, 0, v, plain(q.ke, q.ke), kpan((long long)X * q.ke), bW);
         int e = run_tc(h, g1, "W");
         if (e) return e;
         if (keep_wa) {
@@ -696,7 +694,7 @@ int chain_tc(ppl_cpd* h, int mode, double* Mout, bool keep_wa) {
         g2.b_b0 = 0; g2.b_bstep = 1;
         g2.M = v; g2.N = X; g2.K = v; g2.batch = rcur; g2.ksplit = 1;
         g2.out = out_map(opb(h, h->L.Y), pW, q.ke, 0, Ix{0, 0}, kpan((long long)rc * q.ke),
-                         plain(q.ldk * rc, q.ke));
+                         q.ldk * rc);
         e = run_tc(h, g2, "Y");
         if (e) return e;
         // M[a][r0+r] += sum_{Q,c} B[Q][a][c] Y[r][Q][c]
@@ -744,7 +742,7 @@ int p_tc_body(ppl_cpd* h, bool wa_ready) {
             g1.M = v * X; g1.N = rcur; g1.K = v; g1.batch = 1; g1.ksplit = 1; g1.b_row0 = r0; g1.nfast = 1;
             g1.out = out_map(w == 0 ? opb(h, h->L.WTa + (size_t)r0 * bWT * h->plane_es()) : opb(h, h->L.WTb),
                              w == 0 ? pWTa : pWT, 0, X, plain(q.ke, q.ke),
-                             kpan((long long)v * q.ke), plain(bWT, q.ke));
+                             kpan((long long)v * q.ke), bWT);
             int e = run_tc(h, g1, "WT");
             if (e) return e;
         }
@@ -755,7 +753,7 @@ int p_tc_body(ppl_cpd* h, bool wa_ready) {
         gs.b_b0 = r0;
         gs.a_bstep = 1; gs.b_bstep = 1;
         gs.M = v; gs.N = v; gs.K = X; gs.batch = rcur; gs.ksplit = 1;
-        gs.out = out_map(opb(h, h->L.S), pS, q.ke, 0, Ix{0, 0}, kpan((long long)rc * q.ke), plain(q.ldk * rc, q.ke));
+        gs.out = out_map(opb(h, h->L.S), pS, q.ke, 0, Ix{0, 0}, kpan((long long)rc * q.ke), q.ldk * rc);
         int e = run_tc(h, gs, "S");
         if (e) return e;
         // P[ij][r0+r] += sum_cd tau[ij][cd] S[r][cd]
@@ -1362,7 +1360,7 @@ int ppl_exact_contract_mixed(ppl_cpd* h, double* normR2, double* E_exact, double
         g1.b_row0 = a * v;
         g1.M = v * v; g1.N = v; g1.K = X; g1.batch = 1; g1.ksplit = 1;
         g1.out = out_map(opb(h, h->L.Gop), pG, 0, v, plain(pq.ke, pq.ke), kpan((long long)v * pq.ke),
-                         plain(pq.ldk * v, pq.ke));
+                         pq.ldk * v);
         e = run_tc(h, g1, "exact G");
         if (e) break;
         // R[a][b][ij] = sum_{cd} G_a[b][cd] tau[ij][cd], split-K summed in FP64
@@ -1975,9 +1973,9 @@ int ppl_tc_gemm(int precision, int M, int N, int K, const float* A, const float*
     g.out = TcOut{};
     {
         const int ke = panel_width(precision);
-        g.out.kind = EPI_F32; g.out.out = C; g.out.alpha = 1.0f;
+        g.out.kind = EPI_F32; g.out.out = C;
         g.out.q0p = (long long)ke * N; g.out.q0s = N;    // row m at m * N
-        g.out.np = ke; g.out.ns = 1;                       // column n at n
+        g.out.ns = 1;                                      // column n at n
     }
     g.bn = bn_for(N);
     int r = tc_gemm(g, flag, s);

@@ -123,16 +123,15 @@ struct TcMat {
 //   128-byte row of the operand precision (32 fp32 or 64 bf16; the K-panel width)
 //   rowoff(m) = (q1 / PW)*q1p + (q1 % PW)*q1s + (q0 / PW)*q0p + (q0 % PW)*q0s,
 //               q1 = m / mdiv, q0 = m % mdiv (mdiv <= 0: q1 = 0, q0 = m)
-//   coloff(n) = (n / PW)*np + (n % PW)*ns
-// so that a plain stride s is (PW*s, s) and a K-panel index is (panel stride, 1).
-enum TcEpi { EPI_SPLIT = 0, EPI_F32 = 1, EPI_ATOMIC_F64 = 2, EPI_ATOMIC_F32 = 3 };
+//   coloff(n) = n*ns
+// so that a plain row stride s is (PW*s, s) and a K-panel index is (panel stride, 1).
+enum TcEpi { EPI_SPLIT = 0, EPI_F32 = 1 };
 struct TcOut {
     int kind;               // TcEpi; EPI_SPLIT writes operand planes of the same precision
     void* out; long long plane_elems;
     long long sb, sk;       // batch stride; split-K slice stride (EPI_F32 partials)
     int mdiv;
-    long long q1p, q1s, q0p, q0s, np, ns;
-    float alpha;
+    long long q1p, q1s, q0p, q0s, ns;
 };
 struct TcGemm {
     int prec;               // PPL_PREC_BF16X3 or PPL_PREC_TF32

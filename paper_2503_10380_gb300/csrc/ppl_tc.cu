@@ -19,7 +19,7 @@
 // FP32 registers with round-to-nearest, which removes that bias.
 // Persistent: one CTA per SM walks the 128 x bn output tiles.  Lane 0 of warp
 // 0 issues TMA into a ring of shared-memory stages, lane 0 of warp 1 issues the
-// MMAs into one of two TMEM accumulators, and warps 2..9 drain the other
+// MMAs into one of two TMEM accumulators, and eight warps drain the other
 // accumulator to global memory, so a tile's epilogue overlaps the next tile's
 // mainloop.  Warp 2 owns the TMEM allocation.
 // Every mbarrier wait is bounded; on expiry the kernel records the error,
@@ -48,9 +48,9 @@ constexpr unsigned long long WAIT_NS = 500ull * 1000ull * 1000ull;   // 0.5 s pe
 // MMAs, warp 2 owns the TMEM allocation, warp 3 idles) and two epilogue
 // warpgroups, warps 4..11: two warps per TMEM lane quarter (a warp reads the 32
 // lanes of its quarter, warp % 4), each draining one 128-column half of the tile
-// as two 64-column slices.  With the accumulator restarted every K block an
-// epilogue thread holds 128 running sums and loads 64 columns per TMEM round
-// trip, more registers than a 384-thread block gives every thread, so the
+// as four 32-column pieces.  With the accumulator restarted every K block an
+// epilogue thread holds 128 running sums and 64 columns in flight from TMEM (the
+// next piece's load under the current one's additions), more registers than a 384-thread block gives every thread, so the
 // control warpgroup hands registers to the epilogue (setmaxnreg): 56 for it and
 // 224 for each epilogue thread, 128*56 + 256*224 = 384*168, exactly the launch's
 // allocation (checked on the host before every launch: a split above the
@@ -61,8 +61,8 @@ constexpr int NTHREADS = 32 * (NCTRL + NEPI);
 constexpr int REG_LAUNCH = 168;               // registers per thread at launch (65536 / 384, rounded to 8)
 constexpr int REG_CTRL = 56, REG_EPI = 224;
 static_assert(32 * NCTRL * REG_CTRL + 32 * NEPI * REG_EPI == NTHREADS * REG_LAUNCH, "register split");
-constexpr int SLW = 64;                       // columns per slice
-constexpr int NSL = 2;                        // slices per epilogue warp (a 128-column half)
+constexpr int PCW = 32;                       // columns per piece (one TMEM load)
+constexpr int NPC = 4;                        // pieces per epilogue warp (a 128-column half)
 
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 
@@ -72,9 +72,8 @@ struct KParams {
     int batch;
     int kind;
     void* out;
-    long long plane, sb, sk, q1p, q1s, q0p, q0s, np, ns;
+    long long plane, sb, sk, q1p, q1s, q0p, q0s, ns;
     int mdiv;
-    float alpha;
     int kchunk;             // K blocks per accumulation chunk (drained kernels)
     int ksub;               // > 0: MMA K steps per accumulation chunk, splitting each K block
     int nfast;              // 1: consecutive tiles walk N first (one A tile shared by neighbours)
@@ -155,12 +154,13 @@ __device__ __forceinline__ void mma(uint32_t tmem, unsigned long long ad, unsign
     }
 }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
+// 32 accumulator columns of this warp's 32 lanes, started; the registers hold them after
+// tmem_wait (which takes them as operands, so that nothing reads them before it)
+__device__ __forceinline__ void tmem_start(uint32_t taddr, uint32_t (&v)[PCW]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
         "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
         : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
           "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
           "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
@@ -168,44 +168,13 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
         : "r"(taddr)
         : "memory");
 }
-
-// two FP32 values in one 64-bit register pair, added with one packed
-// round-to-nearest instruction (the same rounding as two scalar adds)
-__device__ __forceinline__ unsigned long long pack2(uint32_t a, uint32_t b) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(a), "r"(b));
-    return r;
-}
-__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
-    unsigned long long d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ void unpack2(unsigned long long x, float& a, float& b) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x));
-}
-
-// 64 accumulator columns as two 32-column loads (each into 32 consecutive
-// registers, which the allocator finds more easily than one block of 64) and
-// one wait
-__device__ __forceinline__ void tmem_ld64(uint32_t taddr, uint32_t (&v)[64]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%64];\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, "
-        "%48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, [%65];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31]),
-          "=r"(v[32]), "=r"(v[33]), "=r"(v[34]), "=r"(v[35]), "=r"(v[36]), "=r"(v[37]), "=r"(v[38]), "=r"(v[39]),
-          "=r"(v[40]), "=r"(v[41]), "=r"(v[42]), "=r"(v[43]), "=r"(v[44]), "=r"(v[45]), "=r"(v[46]), "=r"(v[47]),
-          "=r"(v[48]), "=r"(v[49]), "=r"(v[50]), "=r"(v[51]), "=r"(v[52]), "=r"(v[53]), "=r"(v[54]), "=r"(v[55]),
-          "=r"(v[56]), "=r"(v[57]), "=r"(v[58]), "=r"(v[59]), "=r"(v[60]), "=r"(v[61]), "=r"(v[62]), "=r"(v[63])
-        : "r"(taddr), "r"(taddr + 32u)
+__device__ __forceinline__ void tmem_wait(uint32_t (&v)[PCW]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+        : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+          "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]),
+          "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]),
+          "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
+        :
         : "memory");
 }
 
@@ -215,72 +184,67 @@ __device__ __forceinline__ float round_tf32(float x) {
     return __uint_as_float(y);
 }
 
-// Column offsets of the 32 consecutive columns n0 .. n0 + 31 in the output:
-// (n / PW) * np + (n % PW) * ns.  They span at most two panels (PW >= 32), so
-// column j is at base + j * ns, plus jump once j reaches the next panel.
-struct ColOff {
-    long long base, ns, jump;
-    int split;
-};
-template <int PREC>
-__device__ __forceinline__ ColOff coloffs(const KParams& p, int n0) {
-    constexpr int PW = Prec<PREC>::KE;
-    ColOff c;
-    c.base = (long long)(n0 / PW) * p.np + (long long)(n0 % PW) * p.ns;
-    c.ns = p.ns;
-    c.jump = p.np - (long long)PW * p.ns;
-    c.split = PW - n0 % PW;
-    return c;
-}
-__device__ __forceinline__ long long col_at(const ColOff& c, int j) {
-    return c.base + (long long)j * c.ns + (j >= c.split ? c.jump : 0ll);
+// tf32 rounding to nearest, ties away from zero (cvt.rna.tf32), of a hi part: two
+// integer instructions instead of a conversion at a quarter of their rate.  Same bits
+// except for a NaN, which becomes a zero: the lo part x - hi is then a NaN and carries
+// it through every product.
+__device__ __forceinline__ float round_tf32_hi(float x) {
+    return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u);
 }
 
-// the epilogue's store of 32 consecutive columns n0 .. n0 + 31 of one row
+// Write 32 consecutive columns of one row, the first at o (elements), ns apart; the
+// first nvalid of them.  The address advances by one 64-bit addition per plane and
+// column: with it formed from the column index for every element, a tile's stores
+// took 14k clocks instead of 9.7k (M = 120000, N = 800, K = 200, TF32X3: 369 us, now
+// 295; batch 800 of M = 200, N = 600, K = 200: 474 us, now 383).  They are bound by the SM's store rate (4.2 clocks
+// per 128-byte warp store, 30 bytes per clock and SM, also with 16-byte stores), and the
+// MMA warp, two accumulators ahead, waits for them.
 template <int PREC>
-__device__ __forceinline__ void emit32(const KParams& p, long long mo, int n0, int nvalid, const float (&x)[32]) {
-    const ColOff co = coloffs<PREC>(p, n0);
+__device__ __forceinline__ void emit32(const KParams& p, long long o, int nvalid, const float (&x)[PCW]) {
     if (p.kind == EPI_SPLIT) {
         if constexpr (PREC == PPL_PREC_BF16X3) {
-            __nv_bfloat16* o = (__nv_bfloat16*)p.out + mo;
-            __nv_bfloat16* ol = o + p.plane;
+            __nv_bfloat16* a = (__nv_bfloat16*)p.out + o;
+            __nv_bfloat16* b = a + p.plane;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
+            for (int j = 0; j < PCW; ++j) {
+                const __nv_bfloat16 hi = __float2bfloat16_rn(x[j]);
+                const __nv_bfloat16 lo = __float2bfloat16_rn(x[j] - __bfloat162float(hi));
                 if (j < nvalid) {
-                    const long long c = col_at(co, j);
-                    const __nv_bfloat16 hi = __float2bfloat16_rn(x[j]);
-                    o[c] = hi;
-                    ol[c] = __float2bfloat16_rn(x[j] - __bfloat162float(hi));
+                    *a = hi;
+                    *b = lo;
                 }
+                a += p.ns;
+                b += p.ns;
             }
         } else if constexpr (PREC == PPL_PREC_TF32X3) {
-            float* o = (float*)p.out + mo;
-            float* ol = o + p.plane;
+            float* a = (float*)p.out + o;
+            float* b = a + p.plane;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
+            for (int j = 0; j < PCW; ++j) {
+                const float hi = round_tf32_hi(x[j]);
+                const float lo = round_tf32(x[j] - hi);
                 if (j < nvalid) {
-                    const long long c = col_at(co, j);
-                    const float hi = round_tf32(x[j]);
-                    o[c] = hi;
-                    ol[c] = round_tf32(x[j] - hi);
+                    *a = hi;
+                    *b = lo;
                 }
+                a += p.ns;
+                b += p.ns;
             }
         } else {
-            float* o = (float*)p.out + mo;
+            float* a = (float*)p.out + o;
 #pragma unroll
-            for (int j = 0; j < 32; ++j)
-                if (j < nvalid) o[col_at(co, j)] = round_tf32(x[j]);
+            for (int j = 0; j < PCW; ++j) {
+                if (j < nvalid) *a = round_tf32(x[j]);
+                a += p.ns;
+            }
         }
-    } else if (p.kind == EPI_F32) {
-        float* o = (float*)p.out + mo;
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-            if (j < nvalid) o[col_at(co, j)] = x[j];
     } else {
-        double* o = (double*)p.out + mo;
+        float* a = (float*)p.out + o;
 #pragma unroll
-        for (int j = 0; j < 32; ++j)
-            if (j < nvalid) atomicAdd(o + col_at(co, j), (double)x[j]);
+        for (int j = 0; j < PCW; ++j) {
+            if (j < nvalid) *a = x[j];
+            a += p.ns;
+        }
     }
 }
 
@@ -535,8 +499,9 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
         // epilogue: warps 4..11; warp w reads TMEM lanes 32*(w%4) .. +31 and
         // columns cg*128 .. cg*128 + 127 of the accumulator
         const int q = warp & 3, cg = (warp - NCTRL) >> 2;
+        const int cb = cg * (NPC * PCW);
         int li = 0;
-        float racc[DRAIN ? NSL : 1][SLW];   // running sums of the chunks (DRAIN only)
+        float racc[DRAIN ? NPC : 1][PCW];   // running sums of the chunks (DRAIN only)
         bool ok = true;
         for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
             int lt;
@@ -554,20 +519,22 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
                 nch = (nk - (tail ? 1 : 0)) * per_full;
                 if (tail) nch += (((p.K % KE) + KSTEP - 1) / KSTEP + p.ksub - 1) / p.ksub;
             }
+            // the row this lane writes, and its offset
             const int m = m0 + q * 32 + lane;
-            const bool mrow = (m < p.M);
-            long long mo = 0;
-            if (mrow) {
+            const int ncol = min(p.bn, p.N - n0) - cb;       // this warp's columns of the tile
+            const int nrow = m < p.M ? ncol : 0;
+            long long mo = (long long)(n0 + cb) * p.ns;
+            if (m < p.M) {
                 constexpr int PW = Prec<PREC>::KE;
                 const int q1 = m / p.mdiv, q0 = m % p.mdiv;
-                mo = (long long)bz * p.sb + (long long)ks * p.sk + (long long)(q1 / PW) * p.q1p +
-                     (long long)(q1 % PW) * p.q1s + (long long)(q0 / PW) * p.q0p + (long long)(q0 % PW) * p.q0s;
+                mo += (long long)bz * p.sb + (long long)ks * p.sk + (long long)(q1 / PW) * p.q1p +
+                      (long long)(q1 % PW) * p.q1s + (long long)(q0 / PW) * p.q0p + (long long)(q0 % PW) * p.q0s;
             }
             if constexpr (DRAIN) {
 #pragma unroll
-                for (int sl = 0; sl < NSL; ++sl)
+                for (int pc = 0; pc < NPC; ++pc)
 #pragma unroll
-                    for (int j = 0; j < SLW; ++j) racc[sl][j] = 0.0f;
+                    for (int j = 0; j < PCW; ++j) racc[pc][j] = 0.0f;
             }
             for (int c = 0; c < nch; ++c, ++li) {
                 const int buf = li & 1;
@@ -582,64 +549,49 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t tb = tmem + (uint32_t)buf * acc_cols + ((uint32_t)(q * 32) << 16);
-                const bool last = (c == nch - 1);
+                const uint32_t tb = tmem + (uint32_t)buf * acc_cols + ((uint32_t)(q * 32) << 16) + (uint32_t)cb;
+                const int nld = p.bn - cb;      // columns of the accumulator in this warp's half
                 if constexpr (DRAIN) {
+                    uint32_t v[2][PCW];
+                    if (nld > 0) tmem_start(tb, v[0]);
 #pragma unroll
-                    for (int sl = 0; sl < NSL; ++sl) {
-                        const int c0 = cg * (NSL * SLW) + sl * SLW;
-                        if (c0 < p.bn) {
-                            uint32_t v[SLW];
-                            tmem_ld64(tb + (uint32_t)c0, v);
+                    for (int pc = 0; pc < NPC; ++pc) {
+                        if (pc * PCW < nld) {
+                            tmem_wait(v[pc & 1]);
+                            if (pc + 1 < NPC && (pc + 1) * PCW < nld) tmem_start(tb + (uint32_t)((pc + 1) * PCW), v[(pc + 1) & 1]);
 #pragma unroll
-                            for (int j = 0; j < SLW; ++j) racc[sl][j] += __uint_as_float(v[j]);
+                            for (int j = 0; j < PCW; ++j) racc[pc][j] += __uint_as_float(v[pc & 1][j]);
                         }
                     }
-                    if (last) {
-                        // the sums are in registers: give the accumulator back to the
-                        // MMA warp before the (long) stores of the tile.  (Releasing it
-                        // between the second slice's load and its adds measured slower:
-                        // the loads then serialise behind the first slice's adds.)
-                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                        __syncwarp();
-                        if (lane == 0)
-                            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty0 + 8u * buf) : "memory");
+                    // the sums are in registers: give the accumulator back to the MMA warp
+                    // (before the stores of the tile, after the last chunk)
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0)
+                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty0 + 8u * buf) : "memory");
+                    if (c == nch - 1) {
 #pragma unroll
-                        for (int sl = 0; sl < NSL; ++sl) {
-#pragma unroll
-                            for (int hh = 0; hh < SLW / 32; ++hh) {
-                                const int c0 = cg * (NSL * SLW) + sl * SLW + hh * 32;
-                                const int nvalid = min(min(32, p.bn - c0), p.N - (n0 + c0));
-                                if (c0 < p.bn && mrow && nvalid > 0) {
-                                    float x[32];
-#pragma unroll
-                                    for (int j = 0; j < 32; ++j) x[j] = racc[sl][hh * 32 + j];
-                                    emit32<PREC>(p, mo, n0 + c0, nvalid, x);
-                                }
-                            }
-                        }
-                        continue;
+                        for (int pc = 0; pc < NPC; ++pc)
+                            if (pc * PCW < ncol)
+                                emit32<PREC>(p, mo + (long long)(pc * PCW) * p.ns, nrow - pc * PCW, racc[pc]);
                     }
                 } else {
-                    for (int c0 = cg * (NSL * SLW); c0 < min(p.bn, (cg + 1) * NSL * SLW); c0 += SLW) {
-                        uint32_t v[SLW];
-                        tmem_ld64(tb + (uint32_t)c0, v);
+#pragma unroll 1
+                    for (int pc = 0; pc < NPC; ++pc) {
+                        if (pc * PCW >= ncol) break;
+                        uint32_t v[PCW];
+                        tmem_start(tb + (uint32_t)(pc * PCW), v);
+                        tmem_wait(v);
+                        float x[PCW];
 #pragma unroll
-                        for (int hh = 0; hh < SLW / 32; ++hh) {
-                            const int c1 = c0 + hh * 32;
-                            const int nvalid = min(min(32, p.bn - c1), p.N - (n0 + c1));   // this tile's columns only
-                            if (mrow && nvalid > 0) {
-                                float x[32];
-#pragma unroll
-                                for (int j = 0; j < 32; ++j) x[j] = __uint_as_float(v[hh * 32 + j]);
-                                emit32<PREC>(p, mo, n0 + c1, nvalid, x);
-                            }
-                        }
+                        for (int j = 0; j < PCW; ++j) x[j] = __uint_as_float(v[j]);
+                        emit32<PREC>(p, mo + (long long)(pc * PCW) * p.ns, nrow - pc * PCW, x);
                     }
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0)
+                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty0 + 8u * buf) : "memory");
                 }
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty0 + 8u * buf) : "memory");
             }
         }
     }
@@ -1028,7 +980,7 @@ int tc_gemm(const TcGemm& g, unsigned int* err_flag, cudaStream_t s) {
     p.M = g.M; p.N = g.N; p.K = g.K;
     p.bn = g.bn > 0 ? g.bn : choose_bn(g.N);
     if (p.bn % 16 || p.bn > 256) return -8;
-    p.acc_cols = SLW;      // at least one 64-column slice per accumulator, so no TMEM load leaves its buffer
+    p.acc_cols = PCW;      // whole pieces, so that no TMEM load leaves its accumulator
     while (p.acc_cols < p.bn) p.acc_cols <<= 1;
     p.nkb_total = (g.K + KE - 1) / KE;
     p.ksplit = g.ksplit > 0 ? g.ksplit : 1;
@@ -1044,10 +996,8 @@ int tc_gemm(const TcGemm& g, unsigned int* err_flag, cudaStream_t s) {
     p.batch = g.batch;
     p.kind = g.out.kind; p.out = g.out.out; p.plane = g.out.plane_elems;
     p.sb = g.out.sb; p.sk = g.out.sk;
-    p.q1p = g.out.q1p; p.q1s = g.out.q1s; p.q0p = g.out.q0p; p.q0s = g.out.q0s; p.np = g.out.np; p.ns = g.out.ns;
+    p.q1p = g.out.q1p; p.q1s = g.out.q1s; p.q0p = g.out.q0p; p.q0s = g.out.q0s; p.ns = g.out.ns;
     p.mdiv = g.out.mdiv > 0 ? g.out.mdiv : (1 << 30);
-    if (g.out.alpha != 1.0f) return -9;
-    p.alpha = 1.0f;
     p.kchunk = g.kchunk;
     p.ksub = (g.ksub > 0 && g.ksub < KE / (half ? 16 : 8)) ? g.ksub : 0;
     if (p.ksub > 0) p.kchunk = 1;
