@@ -136,26 +136,71 @@ __device__ __forceinline__ void load_op(uint32_t dst, const CUtensorMap* map, bo
         tma_load_3d(dst, map, kb * ke, row, b, mbar);
 }
 
+// low word of the matrix descriptor of a tile (the high word is the same for every
+// tile); one MMA's K slice further is + 2 (32 bytes)
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return (uint32_t)make_desc(saddr); }
+
+// D (+)= A B^T for one MMA K step; acc != 0 accumulates
 template <int PREC>
-__device__ __forceinline__ void mma(uint32_t tmem, unsigned long long ad, unsigned long long bd, uint32_t idesc,
-                                    uint32_t acc) {
+__device__ __forceinline__ void mma(uint32_t tmem, uint32_t alo, uint32_t blo, uint32_t idesc, uint32_t acc) {
+    const uint32_t dhi = (uint32_t)(make_desc(0) >> 32);
     if constexpr (Prec<PREC>::HALF) {
         asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-            "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+            "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 p, %5, 0;\n\t"
+            "mov.b64 a, {%1, %4};\n\tmov.b64 b, {%2, %4};\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}" ::"r"(tmem),
+            "r"(alo), "r"(blo), "r"(idesc), "r"(dhi), "r"(acc)
             : "memory");
     } else {
         asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-            "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+            "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 p, %5, 0;\n\t"
+            "mov.b64 a, {%1, %4};\n\tmov.b64 b, {%2, %4};\n\t"
+            "tcgen05.mma.cta_group::1.kind::tf32 [%0], a, b, %3, p;\n\t}" ::"r"(tmem),
+            "r"(alo), "r"(blo), "r"(idesc), "r"(dhi), "r"(acc)
             : "memory");
     }
 }
 
-// 32 accumulator columns of this warp's 32 lanes, started; the registers hold them after
-// tmem_wait (which takes them as operands, so that nothing reads them before it)
+// K steps kk0 .. kk1 - 1 of one K block (planes at the descriptor words ah, al, bh, bl).
+// With two planes the small cross products come first, while the accumulator is small,
+// then hi*hi: fewer round-toward-zero additions at full magnitude.
+template <int PREC>
+__device__ __forceinline__ void mma_steps(uint32_t d, uint32_t ah, uint32_t al, uint32_t bh, uint32_t bl, uint32_t idesc,
+                                          int kk0, int kk1, uint32_t acc, uint32_t lofree) {
+    if constexpr (Prec<PREC>::PLANES == 2) {
+        for (int kk = kk0; kk < kk1; ++kk) {
+            mma<PREC>(d, ah + 2u * kk, bl + 2u * kk, idesc, kk > kk0 ? 1u : acc);
+            mma<PREC>(d, al + 2u * kk, bh + 2u * kk, idesc, 1u);
+        }
+        if (lofree) mma_commit(lofree);
+        for (int kk = kk0; kk < kk1; ++kk) mma<PREC>(d, ah + 2u * kk, bh + 2u * kk, idesc, 1u);
+    } else {
+        for (int kk = kk0; kk < kk1; ++kk) mma<PREC>(d, ah + 2u * kk, bh + 2u * kk, idesc, kk > kk0 ? 1u : acc);
+    }
+}
+// A whole K block, unrolled: one thread issues every MMA of the block, and a rolled step
+// loop with 64-bit descriptor arithmetic took it about as long as the MMAs run. Split
+// TF32, 2000 K blocks per CTA and more: M 253 -> 242 us and W 296 -> 275 us at v 200,
+// X 600, R 800; M 2951 -> 2727, W 2981 -> 2820, Y 3334 -> 3108 us at v 600, X 1800, R 480.
+template <int PREC>
+__device__ __forceinline__ void mma_block(uint32_t d, uint32_t ah, uint32_t al, uint32_t bh, uint32_t bl, uint32_t idesc,
+                                          uint32_t acc, uint32_t lofree) {
+    constexpr int NS = Prec<PREC>::KE / Prec<PREC>::KSTEP;
+    if constexpr (Prec<PREC>::PLANES == 2) {
+#pragma unroll
+        for (int kk = 0; kk < NS; ++kk) {
+            mma<PREC>(d, ah + 2u * kk, bl + 2u * kk, idesc, kk > 0 ? 1u : acc);
+            mma<PREC>(d, al + 2u * kk, bh + 2u * kk, idesc, 1u);
+        }
+        mma_commit(lofree);      // the low planes have been read
+#pragma unroll
+        for (int kk = 0; kk < NS; ++kk) mma<PREC>(d, ah + 2u * kk, bh + 2u * kk, idesc, 1u);
+    } else {
+#pragma unroll
+        for (int kk = 0; kk < NS; ++kk) mma<PREC>(d, ah + 2u * kk, bh + 2u * kk, idesc, kk > 0 ? 1u : acc);
+    }
+}
+
 __device__ __forceinline__ void tmem_start(uint32_t taddr, uint32_t (&v)[PCW]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
@@ -263,7 +308,6 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
     constexpr bool SPLIT = (Prec<PREC>::PLANES == 2);
     constexpr int KE = Prec<PREC>::KE;
     constexpr int KSTEP = Prec<PREC>::KSTEP;
-    constexpr int ASTEP_BYTES = 32;           // one MMA's K slice of a 128-byte row
 
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int total = tile0 ? tile0[nprob] : tc_tiles(P[0]);
@@ -287,7 +331,8 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
     const uint32_t bar_off = stage_bytes * S;
     const uint32_t full0 = base + bar_off;
     const uint32_t empty0 = full0 + 8u * S;
-    const uint32_t tfull0 = empty0 + 8u * S;     // 2 accumulators
+    const uint32_t lfree0 = empty0 + 8u * S;     // two planes: the low planes of the stage are free
+    const uint32_t tfull0 = lfree0 + 8u * S;     // 2 accumulators
     const uint32_t tempty0 = tfull0 + 16u;
     const uint32_t drain_bar = tempty0 + 16u;
     const uint32_t slot = drain_bar + 8u;
@@ -303,8 +348,9 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
         s_issued = 0;
         s_consumed = 0;
         for (int s = 0; s < S; ++s) {
-            mbar_init(full0 + 8u * s, 1);
+            mbar_init(full0 + 8u * s, SPLIT ? 2 : 1);
             mbar_init(empty0 + 8u * s, 1);
+            mbar_init(lfree0 + 8u * s, 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(tfull0 + 8u * b, 1);
@@ -333,14 +379,15 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
         if (warp == 0) {
             if (lane == 0) {
                 // TMA producer: one ring of S stages shared by all tiles of this block
-                int it = 0;
+                int it = 0, s = 0;
+                uint32_t ph = 1u;      // parity of the stage's previous use (a first wait passes at once)
                 for (int t = blockIdx.x; t < total && !*vfail; t += gridDim.x) {
                     int lt;
                     const int pi = locate(t, lt);
                     const KParams& p = P[pi];
                     const CUtensorMap* mp = M4 + 4 * pi;
                     const int ntm = (p.M + TM - 1) / TM, ntn = (p.N + p.bn - 1) / p.bn, tiles_mn = ntm * ntn;
-                    const uint32_t tx_bytes = (SPLIT ? 2u : 1u) * (a_bytes + (uint32_t)p.bn * KROW_BYTES);
+                    const uint32_t tx_bytes = a_bytes + (uint32_t)p.bn * KROW_BYTES;   // of one plane
                     const int z = lt / tiles_mn, rem = lt % tiles_mn;
                     const int m0 = (p.nfast ? rem / ntn : rem % ntm) * TM, n0 = (p.nfast ? rem % ntn : rem / ntm) * p.bn;
                     const int bz = z / p.ksplit, ks = z % p.ksplit;
@@ -348,23 +395,39 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
                     const int nk = min(p.per_split, p.nkb_total - kb0);
                     const int a_b = p.a_b0 + bz * p.a_bstep, b_b = p.b_b0 + bz * p.b_bstep;
                     for (int kbi = 0; kbi < nk; ++kbi, ++it) {
-                        const int s = it % S;
-                        if (it >= S && !mbar_wait(empty0 + 8u * s, (uint32_t)((it / S - 1) & 1), wait_ns)) {
+                        const uint32_t sa = base + stage_bytes * s;
+                        const uint32_t fb = full0 + 8u * s;
+                        const int kb = kb0 + kbi;
+                        if constexpr (SPLIT) {
+                            // The low planes are free four MMAs before the high ones, and
+                            // half of a K block is on its way that much earlier: at a width
+                            // of 240 two stages fill shared memory, and the MMA warp waited
+                            // for loads in every block (M at v 600, X 1800, R 480 2727 ->
+                            // 2544 us, W 2820 -> 2678; M at v 200, X 600, R 800 242 -> 225)
+                            if (!mbar_wait(lfree0 + 8u * s, ph, wait_ns)) {
+                                atomicOr(p.err, 1u);
+                                *vfail = 1;
+                                break;
+                            }
+                            mbar_expect_tx(fb, tx_bytes);
+                            load_op(sa + a_bytes, &mp[1], p.a_panel, kb, KE, p.a_row0 + m0, a_b, fb);
+                            load_op(sa + 2u * a_bytes + b_bytes, &mp[3], p.b_panel, kb, KE, p.b_row0 + n0, b_b, fb);
+                            s_issued = it + 1;
+                        }
+                        if (!mbar_wait(empty0 + 8u * s, ph, wait_ns)) {
+                            if constexpr (SPLIT) mbar_arrive(fb);   // no high planes: complete with the low ones
                             atomicOr(p.err, 1u);
                             *vfail = 1;
                             break;
                         }
-                        const uint32_t sa = base + stage_bytes * s;
-                        const uint32_t fb = full0 + 8u * s;
                         mbar_expect_tx(fb, tx_bytes);
-                        const int kb = kb0 + kbi;
                         load_op(sa, &mp[0], p.a_panel, kb, KE, p.a_row0 + m0, a_b, fb);
                         load_op(sa + (SPLIT ? 2u : 1u) * a_bytes, &mp[2], p.b_panel, kb, KE, p.b_row0 + n0, b_b, fb);
-                        if constexpr (SPLIT) {
-                            load_op(sa + a_bytes, &mp[1], p.a_panel, kb, KE, p.a_row0 + m0, a_b, fb);
-                            load_op(sa + 2u * a_bytes + b_bytes, &mp[3], p.b_panel, kb, KE, p.b_row0 + n0, b_b, fb);
-                        }
                         s_issued = it + 1;
+                        if (++s == S) {
+                            s = 0;
+                            ph ^= 1u;
+                        }
                     }
                 }
             }
@@ -372,6 +435,9 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
             if (lane == 0) {
                 // MMA issuer
                 int it = 0, li = 0;   // li counts accumulation chunks (one per tile unless DRAIN)
+                int s = 0;            // stage and parity of its use
+                uint32_t ph = 0u;
+                constexpr int KFULL = KE / KSTEP;
                 bool ok = true;
                 for (int t = blockIdx.x; t < total && ok && !*vfail; t += gridDim.x) {
                     int lt;
@@ -387,8 +453,7 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
                     if (DRAIN && p.ksub > 0) {
                         // each K block in chunks of ksub MMA K steps, one accumulator each
                         for (int kbi = 0; kbi < nk && ok; ++kbi, ++it) {
-                            const int s = it % S;
-                            if (!mbar_wait(full0 + 8u * s, (uint32_t)((it / S) & 1), wait_ns)) {
+                            if (!mbar_wait(full0 + 8u * s, ph, wait_ns)) {
                                 atomicOr(p.err, 2u);
                                 *vfail = 1;
                                 ok = false;
@@ -396,15 +461,12 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
                             }
                             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                             const uint32_t sa = base + stage_bytes * s;
-                            const uint32_t sah = sa, sal = sa + a_bytes;
-                            const uint32_t sbh = sa + (SPLIT ? 2u : 1u) * a_bytes, sbl = sbh + b_bytes;
-                            const int kc = (kb0 + kbi) * KE;
-                            int ksteps = KE / KSTEP;
-                            if (p.K - kc < KE) ksteps = (p.K - kc + KSTEP - 1) / KSTEP;
-                            const unsigned long long dah = make_desc(sah), dbh = make_desc(sbh);
-                            const unsigned long long dal = make_desc(sal), dbl = make_desc(sbl);
+                            const uint32_t ah = desc_lo(sa), al = desc_lo(sa + a_bytes);
+                            const uint32_t sb = sa + (SPLIT ? 2u : 1u) * a_bytes;
+                            const uint32_t bh = desc_lo(sb), bl = desc_lo(sb + b_bytes);
+                            const int kleft = p.K - (kb0 + kbi) * KE;
+                            const int ksteps = min(KFULL, (kleft + KSTEP - 1) / KSTEP);
                             for (int kk0 = 0; kk0 < ksteps; kk0 += p.ksub, ++li) {
-                                const int kk1 = min(ksteps, kk0 + p.ksub);
                                 const int buf = li & 1;
                                 if (li >= 2 && !mbar_wait(tempty0 + 8u * buf, (uint32_t)(((li >> 1) - 1) & 1), wait_ns)) {
                                     atomicOr(p.err, 8u);
@@ -413,28 +475,18 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
                                     break;
                                 }
                                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                                const uint32_t d = tmem + (uint32_t)buf * acc_cols;
-                                if constexpr (SPLIT) {
-                                    for (int kk = kk0; kk < kk1; ++kk) {
-                                        const unsigned long long off = (unsigned long long)((kk * ASTEP_BYTES) >> 4);
-                                        mma<PREC>(d, dah + off, dbl + off, idesc, kk > kk0 ? 1u : 0u);
-                                        mma<PREC>(d, dal + off, dbh + off, idesc, 1u);
-                                    }
-                                    for (int kk = kk0; kk < kk1; ++kk) {
-                                        const unsigned long long off = (unsigned long long)((kk * ASTEP_BYTES) >> 4);
-                                        mma<PREC>(d, dah + off, dbh + off, idesc, 1u);
-                                    }
-                                } else {
-                                    for (int kk = kk0; kk < kk1; ++kk) {
-                                        const unsigned long long off = (unsigned long long)((kk * ASTEP_BYTES) >> 4);
-                                        mma<PREC>(d, dah + off, dbh + off, idesc, kk > kk0 ? 1u : 0u);
-                                    }
-                                }
+                                mma_steps<PREC>(tmem + (uint32_t)buf * acc_cols, ah, al, bh, bl, idesc, kk0,
+                                                min(ksteps, kk0 + p.ksub), 0u, 0u);
                                 mma_commit(tfull0 + 8u * buf);
                             }
                             if (!ok) break;
+                            if constexpr (SPLIT) mma_commit(lfree0 + 8u * s);
                             mma_commit(empty0 + 8u * s);
                             s_consumed = it + 1;
+                            if (++s == S) {
+                                s = 0;
+                                ph ^= 1u;
+                            }
                         }
                         continue;
                     }
@@ -450,8 +502,7 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         const uint32_t d = tmem + (uint32_t)buf * acc_cols;
                         for (int kbi = kc0; kbi < kc1; ++kbi, ++it) {
-                            const int s = it % S;
-                            if (!mbar_wait(full0 + 8u * s, (uint32_t)((it / S) & 1), wait_ns)) {
+                            if (!mbar_wait(full0 + 8u * s, ph, wait_ns)) {
                                 atomicOr(p.err, 2u);
                                 *vfail = 1;
                                 ok = false;
@@ -459,33 +510,21 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
                             }
                             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                             const uint32_t sa = base + stage_bytes * s;
-                            const uint32_t sah = sa, sal = sa + a_bytes;
-                            const uint32_t sbh = sa + (SPLIT ? 2u : 1u) * a_bytes, sbl = sbh + b_bytes;
-                            const int kc = (kb0 + kbi) * KE;
-                            int ksteps = KE / KSTEP;
-                            if (p.K - kc < KE) ksteps = (p.K - kc + KSTEP - 1) / KSTEP;
-                            const unsigned long long dah = make_desc(sah), dbh = make_desc(sbh);
-                            const unsigned long long dal = make_desc(sal), dbl = make_desc(sbl);
-                            if constexpr (SPLIT) {
-                                // the small cross products first, while the accumulator is small,
-                                // then hi*hi: fewer round-toward-zero additions at full magnitude
-                                for (int kk = 0; kk < ksteps; ++kk) {
-                                    const unsigned long long off = (unsigned long long)((kk * ASTEP_BYTES) >> 4);
-                                    mma<PREC>(d, dah + off, dbl + off, idesc, (kbi > kc0 || kk > 0) ? 1u : 0u);
-                                    mma<PREC>(d, dal + off, dbh + off, idesc, 1u);
-                                }
-                                for (int kk = 0; kk < ksteps; ++kk) {
-                                    const unsigned long long off = (unsigned long long)((kk * ASTEP_BYTES) >> 4);
-                                    mma<PREC>(d, dah + off, dbh + off, idesc, 1u);
-                                }
-                            } else {
-                                for (int kk = 0; kk < ksteps; ++kk) {
-                                    const unsigned long long off = (unsigned long long)((kk * ASTEP_BYTES) >> 4);
-                                    mma<PREC>(d, dah + off, dbh + off, idesc, (kbi > kc0 || kk > 0) ? 1u : 0u);
-                                }
-                            }
+                            const uint32_t ah = desc_lo(sa), al = desc_lo(sa + a_bytes);
+                            const uint32_t sb = sa + (SPLIT ? 2u : 1u) * a_bytes;
+                            const uint32_t bh = desc_lo(sb), bl = desc_lo(sb + b_bytes);
+                            const int kleft = p.K - (kb0 + kbi) * KE;
+                            const uint32_t acc = kbi > kc0 ? 1u : 0u;
+                            if (kleft >= KE)
+                                mma_block<PREC>(d, ah, al, bh, bl, idesc, acc, lfree0 + 8u * s);
+                            else
+                                mma_steps<PREC>(d, ah, al, bh, bl, idesc, 0, (kleft + KSTEP - 1) / KSTEP, acc, lfree0 + 8u * s);
                             mma_commit(empty0 + 8u * s);
                             s_consumed = it + 1;
+                            if (++s == S) {
+                                s = 0;
+                                ph ^= 1u;
+                            }
                         }
                         if (!ok) break;
                         mma_commit(tfull0 + 8u * buf);
@@ -1022,7 +1061,7 @@ int tc_gemm(const TcGemm& g, unsigned int* err_flag, cudaStream_t s) {
         mBl = mBh;
     }
     a.p = p;
-    const size_t smem = (size_t)stage_bytes * p.stages + 1024 + 16 * p.stages + 64;
+    const size_t smem = (size_t)stage_bytes * p.stages + 1024 + 24 * p.stages + 64;
     if (smem > (size_t)SMEM_ATTR) return -6;
     const long long tiles = (long long)((g.M + TM - 1) / TM) * ((g.N + p.bn - 1) / p.bn) * g.batch * p.ksplit;
     if (tiles > (1ll << 30)) return -4;
@@ -1174,7 +1213,7 @@ int tc_group_node_params(const void* f, const void* const* args, int n, cudaKern
     const int stage_bytes = planes * (TM + a.bn_max) * KROW_BYTES;
     a.stages = SMEM_BUDGET / stage_bytes;
     if (a.stages > 8) a.stages = 8;
-    const size_t smem = (size_t)stage_bytes * a.stages + 1024 + 16 * a.stages + 64;
+    const size_t smem = (size_t)stage_bytes * a.stages + 1024 + 24 * a.stages + 64;
     if (a.stages < 2 || smem > (size_t)SMEM_ATTR) {
         delete g;
         return -6;
