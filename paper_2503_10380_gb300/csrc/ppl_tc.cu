@@ -41,8 +41,8 @@ namespace {
 
 constexpr int TM = 128;               // rows of the accumulator tile (TMEM lanes)
 constexpr int KROW_BYTES = 128;       // one swizzle row: 64 bf16 or 32 fp32
-constexpr int SMEM_BUDGET = 200 * 1024;      // operand stages
-constexpr int SMEM_ATTR = 220 * 1024;        // dynamic smem opt-in (stages + alignment + barriers)
+constexpr int SMEM_BUDGET = 222 * 1024;      // operand stages
+constexpr int SMEM_ATTR = 226 * 1024;        // dynamic smem opt-in (stages + alignment + barriers)
 constexpr unsigned long long WAIT_NS = 500ull * 1000ull * 1000ull;   // 0.5 s per wait
 // Block layout: one control warpgroup (warp 0 issues TMA, warp 1 issues the
 // MMAs, warp 2 owns the TMEM allocation, warp 3 idles) and two epilogue
@@ -63,6 +63,23 @@ constexpr int REG_CTRL = 56, REG_EPI = 224;
 static_assert(32 * NCTRL * REG_CTRL + 32 * NEPI * REG_EPI == NTHREADS * REG_LAUNCH, "register split");
 constexpr int PCW = 32;                       // columns per piece (one TMEM load)
 constexpr int NPC = 4;                        // pieces per epilogue warp (a 128-column half)
+// With restarted accumulation the warps that sum the chunks cannot also write the tile
+// while the next one is multiplied: their sums fill the registers, and a 128 x 256 tile
+// (245 KB of two-plane output) leaves the SM at 30 bytes per clock, the time of four to
+// five K blocks, during which the MMA warp runs out of accumulators.  The handed-over
+// form (HAND), for short K, splits the two jobs: tiles are at most 160 columns wide, so
+// that TMEM holds a third buffer next to the two accumulators; the eight summing warps
+// (80 columns each) put a finished tile there and go on with the next one, while four
+// more warps read it and write it out.
+// 16 warps: 128 * 56 + 256 * 168 + 128 * 120 = 512 * 128 registers.
+constexpr int HBN = 160;                      // widest N tile of the handed-over form
+constexpr int HKB = 8;                        // most K blocks of a handed-over contraction
+constexpr int HPW = 16;                       // columns per piece of a summing warp
+constexpr int HNP = HBN / 2 / HPW;            // pieces per summing warp
+constexpr int NSTORE = 4;                     // storing warps, one per TMEM lane quarter
+constexpr int HTHREADS = NTHREADS + 32 * NSTORE;
+constexpr int HREG_LAUNCH = 128, HREG_SUM = 168, HREG_STORE = 120;
+static_assert(32 * NCTRL * REG_CTRL + 32 * NEPI * HREG_SUM + 32 * NSTORE * HREG_STORE == HTHREADS * HREG_LAUNCH, "register split");
 
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 
@@ -229,6 +246,34 @@ __device__ __forceinline__ float round_tf32(float x) {
     return __uint_as_float(y);
 }
 
+// the same for 16 columns
+__device__ __forceinline__ void tmem_start16(uint32_t taddr, uint32_t (&v)[HPW]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_wait16(uint32_t (&v)[HPW]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+        : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+          "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])
+        :
+        : "memory");
+}
+// 16 columns of this warp's lanes into TMEM (complete after tmem_stored)
+__device__ __forceinline__ void tmem_put16(uint32_t taddr, const float (&x)[HPW]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(taddr),
+          "r"(__float_as_uint(x[0])), "r"(__float_as_uint(x[1])), "r"(__float_as_uint(x[2])), "r"(__float_as_uint(x[3])), "r"(__float_as_uint(x[4])), "r"(__float_as_uint(x[5])),
+          "r"(__float_as_uint(x[6])), "r"(__float_as_uint(x[7])), "r"(__float_as_uint(x[8])), "r"(__float_as_uint(x[9])), "r"(__float_as_uint(x[10])),
+          "r"(__float_as_uint(x[11])), "r"(__float_as_uint(x[12])), "r"(__float_as_uint(x[13])), "r"(__float_as_uint(x[14])), "r"(__float_as_uint(x[15]))
+        : "memory");
+}
+__device__ __forceinline__ void tmem_stored() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // tf32 rounding to nearest, ties away from zero (cvt.rna.tf32), of a hi part: two
 // integer instructions instead of a conversion at a quarter of their rate.  Same bits
 // except for a NaN, which becomes a zero: the lo part x - hi is then a NaN and carries
@@ -293,6 +338,15 @@ __device__ __forceinline__ void emit32(const KParams& p, long long o, int nvalid
     }
 }
 
+// output offset of row m in batch entry bz, split-K slice ks
+template <int PREC>
+__device__ __forceinline__ long long row_offset(const KParams& p, int m, int bz, int ks) {
+    constexpr int PW = Prec<PREC>::KE;
+    const int q1 = m / p.mdiv, q0 = m % p.mdiv;
+    return (long long)bz * p.sb + (long long)ks * p.sk + (long long)(q1 / PW) * p.q1p + (long long)(q1 % PW) * p.q1s +
+           (long long)(q0 / PW) * p.q0p + (long long)(q0 % PW) * p.q0s;
+}
+
 // tiles of one contraction
 __host__ __device__ __forceinline__ int tc_tiles(const KParams& p) {
     return ((p.M + TM - 1) / TM) * ((p.N + p.bn - 1) / p.bn) * p.batch * p.ksplit;
@@ -302,7 +356,7 @@ __host__ __device__ __forceinline__ int tc_tiles(const KParams& p) {
 // of contraction i, whose tiles are tile0[i] .. tile0[i + 1] - 1 of the walk
 // (tile0 == nullptr: one contraction).  Stages of bn_max-wide B tiles, S of them,
 // and two TMEM accumulators of acc_cols_u columns serve every contraction.
-template <int PREC, bool DRAIN>
+template <int PREC, bool DRAIN, bool HAND>
 __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4, const int* tile0, int nprob,
                                         int bn_max, int S, int acc_cols_u, unsigned long long wait_ns) {
     constexpr bool SPLIT = (Prec<PREC>::PLANES == 2);
@@ -335,13 +389,21 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
     const uint32_t tfull0 = lfree0 + 8u * S;     // 2 accumulators
     const uint32_t tempty0 = tfull0 + 16u;
     const uint32_t drain_bar = tempty0 + 16u;
-    const uint32_t slot = drain_bar + 8u;
+    const uint32_t sfull = drain_bar + 8u;       // HAND: the third TMEM buffer holds a tile
+    const uint32_t sempty = sfull + 8u;          // HAND: it has been read
+    const uint32_t slot = sempty + 8u;
     volatile uint32_t* slot_ptr = (volatile uint32_t*)(gbase + (slot - base));
     __shared__ int s_fail;
     __shared__ int s_issued, s_consumed;
 
     const uint32_t acc_cols = (uint32_t)acc_cols_u;
-    const uint32_t ncols = 2u * acc_cols;
+    // columns allocated (a power of two), and the third buffer behind the accumulators
+    uint32_t ncols = 2u * acc_cols;
+    const uint32_t scol = ncols;
+    if constexpr (HAND) {
+        ncols = 32u;
+        while (ncols < 3u * acc_cols) ncols <<= 1;
+    }
 
     if (threadIdx.x == 0) {
         s_fail = 0;
@@ -357,6 +419,8 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
             mbar_init(tempty0 + 8u * b, NEPI);
         }
         mbar_init(drain_bar, 1);
+        mbar_init(sfull, NEPI);
+        mbar_init(sempty, NSTORE);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)&M4[0]) : "memory");
@@ -533,6 +597,115 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
                 mma_commit(drain_bar);   // completes once every MMA issued here has finished
             }
         }
+    } else if (HAND && warp >= NCTRL + NEPI) {
+        if constexpr (HAND) {
+            asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(HREG_STORE) : "memory");
+            // storing warps 12..15: warp w writes TMEM lanes 32*(w%4) .. +31 of every tile
+            const int q = warp & 3;
+            int nt = 0;
+            for (int t = blockIdx.x; t < total; t += gridDim.x, ++nt) {
+                int lt;
+                const KParams& p = P[locate(t, lt)];
+                const int ntm = (p.M + TM - 1) / TM, ntn = (p.N + p.bn - 1) / p.bn, tiles_mn = ntm * ntn;
+                const int z = lt / tiles_mn, rem = lt % tiles_mn;
+                const int m0 = (p.nfast ? rem / ntn : rem % ntm) * TM, n0 = (p.nfast ? rem % ntn : rem / ntm) * p.bn;
+                const int bz = z / p.ksplit, ks = z % p.ksplit;
+                const int m = m0 + q * 32 + lane;
+                const int ncol = min(p.bn, p.N - n0), nrow = m < p.M ? ncol : 0;
+                const long long mo = (long long)n0 * p.ns + (m < p.M ? row_offset<PREC>(p, m, bz, ks) : 0);
+                if (!mbar_wait(sfull, (uint32_t)(nt & 1), wait_ns)) {
+                    if (lane == 0) atomicOr(p.err, 4u);
+                    *vfail = 1;
+                    break;
+                }
+                if (*vfail) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t tb = tmem + scol + ((uint32_t)(q * 32) << 16);
+                const int npc = (ncol + PCW - 1) / PCW;
+#pragma unroll 1
+                for (int pc = 0; pc < npc; ++pc) {
+                    uint32_t v[PCW];
+                    tmem_start(tb + (uint32_t)(pc * PCW), v);
+                    tmem_wait(v);
+                    if (pc == npc - 1) {       // the buffer has been read
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(sempty);
+                    }
+                    float x[PCW];
+#pragma unroll
+                    for (int j = 0; j < PCW; ++j) x[j] = __uint_as_float(v[j]);
+                    emit32<PREC>(p, mo + (long long)(pc * PCW) * p.ns, nrow - pc * PCW, x);
+                }
+            }
+        }
+    } else if constexpr (HAND) {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(HREG_SUM) : "memory");
+        // summing warps 4..11: warp w reads TMEM lanes 32*(w%4) .. +31 and one half of the
+        // accumulator's columns (a multiple of 16)
+        const int q = warp & 3, cg = (warp - NCTRL) >> 2;
+        int li = 0, nt = 0;
+        bool ok = true;
+        float racc[HNP][HPW];
+        for (int t = blockIdx.x; t < total && ok; t += gridDim.x, ++nt) {
+            int lt;
+            const KParams& p = P[locate(t, lt)];
+            const int tiles_mn = ((p.M + TM - 1) / TM) * ((p.N + p.bn - 1) / p.bn);
+            const int ks = lt / tiles_mn % p.ksplit;
+            const int nk = min(p.per_split, p.nkb_total - ks * p.per_split);
+            const int nch = (nk + p.kchunk - 1) / p.kchunk;
+            const int half = (p.bn / HPW + 1) / 2 * HPW;
+            const int cb = cg * half, nld = cg ? p.bn - half : half;
+#pragma unroll
+            for (int pc = 0; pc < HNP; ++pc)
+#pragma unroll
+                for (int j = 0; j < HPW; ++j) racc[pc][j] = 0.0f;
+            for (int c = 0; c < nch; ++c, ++li) {
+                const int buf = li & 1;
+                if (!mbar_wait(tfull0 + 8u * buf, (uint32_t)((li >> 1) & 1), wait_ns)) {
+                    if (lane == 0) atomicOr(p.err, 4u);
+                    *vfail = 1;
+                    ok = false;
+                    break;
+                }
+                if (*vfail) {
+                    ok = false;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t tb = tmem + (uint32_t)buf * acc_cols + ((uint32_t)(q * 32) << 16) + (uint32_t)cb;
+                uint32_t v[2][HPW];
+                if (nld > 0) tmem_start16(tb, v[0]);
+#pragma unroll
+                for (int pc = 0; pc < HNP; ++pc) {
+                    if (pc * HPW < nld) {
+                        tmem_wait16(v[pc & 1]);
+                        if (pc + 1 < HNP && (pc + 1) * HPW < nld) tmem_start16(tb + (uint32_t)((pc + 1) * HPW), v[(pc + 1) & 1]);
+#pragma unroll
+                        for (int j = 0; j < HPW; ++j) racc[pc][j] += __uint_as_float(v[pc & 1][j]);
+                    }
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(tempty0 + 8u * buf);
+            }
+            if (!ok) break;
+            // hand the tile over, once the previous one has been read
+            if (nt > 0 && !mbar_wait(sempty, (uint32_t)((nt - 1) & 1), wait_ns)) {
+                if (lane == 0) atomicOr(p.err, 4u);
+                *vfail = 1;
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t ts = tmem + scol + ((uint32_t)(q * 32) << 16) + (uint32_t)cb;
+#pragma unroll
+            for (int pc = 0; pc < HNP; ++pc)
+                if (pc * HPW < nld) tmem_put16(ts + (uint32_t)(pc * HPW), racc[pc]);
+            tmem_stored();
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(sfull);
+        }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REG_EPI) : "memory");
         // epilogue: warps 4..11; warp w reads TMEM lanes 32*(w%4) .. +31 and
@@ -562,13 +735,7 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
             const int m = m0 + q * 32 + lane;
             const int ncol = min(p.bn, p.N - n0) - cb;       // this warp's columns of the tile
             const int nrow = m < p.M ? ncol : 0;
-            long long mo = (long long)(n0 + cb) * p.ns;
-            if (m < p.M) {
-                constexpr int PW = Prec<PREC>::KE;
-                const int q1 = m / p.mdiv, q0 = m % p.mdiv;
-                mo += (long long)bz * p.sb + (long long)ks * p.sk + (long long)(q1 / PW) * p.q1p +
-                      (long long)(q1 % PW) * p.q1s + (long long)(q0 / PW) * p.q0p + (long long)(q0 % PW) * p.q0s;
-            }
+            const long long mo = (long long)(n0 + cb) * p.ns + (m < p.M ? row_offset<PREC>(p, m, bz, ks) : 0);
             if constexpr (DRAIN) {
 #pragma unroll
                 for (int pc = 0; pc < NPC; ++pc)
@@ -607,7 +774,7 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
                     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                     __syncwarp();
                     if (lane == 0)
-                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty0 + 8u * buf) : "memory");
+                        mbar_arrive(tempty0 + 8u * buf);
                     if (c == nch - 1) {
 #pragma unroll
                         for (int pc = 0; pc < NPC; ++pc)
@@ -629,7 +796,7 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
                     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                     __syncwarp();
                     if (lane == 0)
-                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty0 + 8u * buf) : "memory");
+                        mbar_arrive(tempty0 + 8u * buf);
                 }
             }
         }
@@ -653,24 +820,31 @@ __device__ __forceinline__ void tc_body(const KParams* P, const CUtensorMap* M4,
     }
 }
 
-template <int PREC, bool DRAIN>
-__global__ void __launch_bounds__(NTHREADS, 1) k_tc_gemm(const __grid_constant__ TcArgs a) {
-    tc_body<PREC, DRAIN>(&a.p, a.m, nullptr, 1, a.p.bn, a.p.stages, a.p.acc_cols, a.p.wait_ns);
+// MODE: 0 one accumulator per tile, 1 restarted, 2 restarted with the tiles handed over
+constexpr int threads_of(int mode) { return mode == 2 ? HTHREADS : NTHREADS; }
+
+template <int PREC, int MODE>
+__global__ void __launch_bounds__(threads_of(MODE), 1) k_tc_gemm(const __grid_constant__ TcArgs a) {
+    tc_body<PREC, MODE != 0, MODE == 2>(&a.p, a.m, nullptr, 1, a.p.bn, a.p.stages, a.p.acc_cols, a.p.wait_ns);
 }
 
-template <int PREC, bool DRAIN>
-__global__ void __launch_bounds__(NTHREADS, 1) k_tc_gemm_group(const __grid_constant__ TcGroupArgs g) {
-    tc_body<PREC, DRAIN>(g.p, &g.m[0][0], g.tile0, g.n, g.bn_max, g.stages, g.acc_cols, g.wait_ns);
+template <int PREC, int MODE>
+__global__ void __launch_bounds__(threads_of(MODE), 1) k_tc_gemm_group(const __grid_constant__ TcGroupArgs g) {
+    tc_body<PREC, MODE != 0, MODE == 2>(g.p, &g.m[0][0], g.tile0, g.n, g.bn_max, g.stages, g.acc_cols, g.wait_ns);
 }
 
-// the single-contraction kernels and their grouped counterparts
-const void* const k_single[6] = {(const void*)k_tc_gemm<PPL_PREC_BF16X3, false>, (const void*)k_tc_gemm<PPL_PREC_BF16X3, true>,
-                                 (const void*)k_tc_gemm<PPL_PREC_TF32, false>,   (const void*)k_tc_gemm<PPL_PREC_TF32, true>,
-                                 (const void*)k_tc_gemm<PPL_PREC_TF32X3, false>, (const void*)k_tc_gemm<PPL_PREC_TF32X3, true>};
-const void* const k_grouped[6] = {
-    (const void*)k_tc_gemm_group<PPL_PREC_BF16X3, false>, (const void*)k_tc_gemm_group<PPL_PREC_BF16X3, true>,
-    (const void*)k_tc_gemm_group<PPL_PREC_TF32, false>,   (const void*)k_tc_gemm_group<PPL_PREC_TF32, true>,
-    (const void*)k_tc_gemm_group<PPL_PREC_TF32X3, false>, (const void*)k_tc_gemm_group<PPL_PREC_TF32X3, true>};
+// the single-contraction kernels and their grouped counterparts: 3 * precision + mode
+constexpr int NKERN = 9;
+const void* const k_single[NKERN] = {
+    (const void*)k_tc_gemm<PPL_PREC_BF16X3, 0>, (const void*)k_tc_gemm<PPL_PREC_BF16X3, 1>, (const void*)k_tc_gemm<PPL_PREC_BF16X3, 2>,
+    (const void*)k_tc_gemm<PPL_PREC_TF32, 0>,   (const void*)k_tc_gemm<PPL_PREC_TF32, 1>,   (const void*)k_tc_gemm<PPL_PREC_TF32, 2>,
+    (const void*)k_tc_gemm<PPL_PREC_TF32X3, 0>, (const void*)k_tc_gemm<PPL_PREC_TF32X3, 1>, (const void*)k_tc_gemm<PPL_PREC_TF32X3, 2>};
+const void* const k_grouped[NKERN] = {
+    (const void*)k_tc_gemm_group<PPL_PREC_BF16X3, 0>, (const void*)k_tc_gemm_group<PPL_PREC_BF16X3, 1>,
+    (const void*)k_tc_gemm_group<PPL_PREC_BF16X3, 2>, (const void*)k_tc_gemm_group<PPL_PREC_TF32, 0>,
+    (const void*)k_tc_gemm_group<PPL_PREC_TF32, 1>,   (const void*)k_tc_gemm_group<PPL_PREC_TF32, 2>,
+    (const void*)k_tc_gemm_group<PPL_PREC_TF32X3, 0>, (const void*)k_tc_gemm_group<PPL_PREC_TF32X3, 1>,
+    (const void*)k_tc_gemm_group<PPL_PREC_TF32X3, 2>};
 
 // Sum split-K partials part[ks][n][m] (fp32) in FP64 into out[m * ldo + n].
 __global__ void k_reduce_partials(const float* part, int ksplit, int M, int N, double* out, long long ldo) {
@@ -964,12 +1138,9 @@ int tc_init_driver() {
     g_encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
     static bool attr_done = false;
     if (!attr_done) {
-        const void* fns[12];
-        for (int i = 0; i < 6; ++i) {
-            fns[i] = k_single[i];
-            fns[6 + i] = k_grouped[i];
-        }
-        for (const void* f : fns) {
+        for (int i = 0; i < 2 * NKERN; ++i) {
+            const void* f = i < NKERN ? k_single[i] : k_grouped[i - NKERN];
+            const int mode = i % NKERN % 3;
             if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_ATTR) != cudaSuccess) {
                 cudaGetLastError();
                 return -2;
@@ -981,7 +1152,7 @@ int tc_init_driver() {
                 cudaGetLastError();
                 return -2;
             }
-            if (fa.numRegs != REG_LAUNCH || fa.maxThreadsPerBlock < NTHREADS) return -12;
+            if (fa.numRegs != (mode == 2 ? HREG_LAUNCH : REG_LAUNCH) || fa.maxThreadsPerBlock < threads_of(mode)) return -12;
         }
         attr_done = true;
     }
@@ -991,13 +1162,14 @@ int tc_init_driver() {
 namespace {
 
 template <int PREC>
-void launch_tc(bool drain, int grid, size_t smem, cudaStream_t s, const TcArgs& a) {
-    if (drain)
-        k_tc_gemm<PREC, true><<<grid, NTHREADS, smem, s>>>(a);
+void launch_tc(int mode, int grid, size_t smem, cudaStream_t s, const TcArgs& a) {
+    if (mode == 2)
+        k_tc_gemm<PREC, 2><<<grid, HTHREADS, smem, s>>>(a);
+    else if (mode == 1)
+        k_tc_gemm<PREC, 1><<<grid, NTHREADS, smem, s>>>(a);
     else
-        k_tc_gemm<PREC, false><<<grid, NTHREADS, smem, s>>>(a);
+        k_tc_gemm<PREC, 0><<<grid, NTHREADS, smem, s>>>(a);
 }
-
 
 }  // namespace
 
@@ -1019,13 +1191,29 @@ int tc_gemm(const TcGemm& g, unsigned int* err_flag, cudaStream_t s) {
     p.M = g.M; p.N = g.N; p.K = g.K;
     p.bn = g.bn > 0 ? g.bn : choose_bn(g.N);
     if (p.bn % 16 || p.bn > 256) return -8;
-    p.acc_cols = PCW;      // whole pieces, so that no TMEM load leaves its accumulator
-    while (p.acc_cols < p.bn) p.acc_cols <<= 1;
     p.nkb_total = (g.K + KE - 1) / KE;
     p.ksplit = g.ksplit > 0 ? g.ksplit : 1;
     if (p.ksplit > p.nkb_total) p.ksplit = p.nkb_total;
     p.per_split = (p.nkb_total + p.ksplit - 1) / p.ksplit;
     p.ksplit = (p.nkb_total + p.per_split - 1) / p.per_split;   // every split slice is non-empty
+    p.ksub = (g.ksub > 0 && g.ksub < KE / (half ? 16 : 8)) ? g.ksub : 0;
+    p.kchunk = p.ksub > 0 ? 1 : g.kchunk;
+    // Restarted accumulation hands its tiles over where K is so short that writing them
+    // is what the time goes to.  Split TF32, wide tiles -> handed over: 7 K blocks (v 200,
+    // X 600, R 800) W 278 -> 242 us, Y 362 -> 359; 8 (251, 773, 605) W 418 -> 415, Y 439
+    // -> 397.  From 13 on the narrower tiles' loads cost more: W 692 -> 721, Y 789 -> 864
+    // (400, 1000, 400), and at 19 W 2678 -> 2779, Y 2977 -> 3111 (600, 1800, 480).
+    // Split-K partials keep the wide tiles: their K is long.
+    const bool drain = p.ksub > 0 || (g.kchunk > 0 && g.kchunk < p.per_split);
+    const int mode = !drain ? 0 : (g.out.kind == EPI_SPLIT && p.ksub == 0 && p.nkb_total <= HKB) ? 2 : 1;
+    if (mode == 2) {
+        const int nt = (g.N + HBN - 1) / HBN;
+        p.bn = ((g.N + nt - 1) / nt + 15) / 16 * 16;
+        p.acc_cols = p.bn;
+    } else {
+        p.acc_cols = PCW;      // whole pieces, so that no TMEM load leaves its accumulator
+        while (p.acc_cols < p.bn) p.acc_cols <<= 1;
+    }
     const int stage_bytes = (split ? 2 : 1) * (TM + p.bn) * KROW_BYTES;
     p.stages = SMEM_BUDGET / stage_bytes;
     if (p.stages > 8) p.stages = 8;
@@ -1037,14 +1225,9 @@ int tc_gemm(const TcGemm& g, unsigned int* err_flag, cudaStream_t s) {
     p.sb = g.out.sb; p.sk = g.out.sk;
     p.q1p = g.out.q1p; p.q1s = g.out.q1s; p.q0p = g.out.q0p; p.q0s = g.out.q0s; p.ns = g.out.ns;
     p.mdiv = g.out.mdiv > 0 ? g.out.mdiv : (1 << 30);
-    p.kchunk = g.kchunk;
-    p.ksub = (g.ksub > 0 && g.ksub < KE / (half ? 16 : 8)) ? g.ksub : 0;
-    if (p.ksub > 0) p.kchunk = 1;
     p.nfast = g.nfast;
     p.a_panel = g.A.panel ? 1 : 0;
     p.b_panel = g.B.panel ? 1 : 0;
-    const bool drain = p.ksub > 0 || (g.kchunk > 0 && g.kchunk < p.per_split);
-    if (drain && p.bn > 256) return -8;
     p.err = err_flag;
     p.wait_ns = g.wait_ns > 0 ? g.wait_ns : WAIT_NS;
 
@@ -1061,18 +1244,18 @@ int tc_gemm(const TcGemm& g, unsigned int* err_flag, cudaStream_t s) {
         mBl = mBh;
     }
     a.p = p;
-    const size_t smem = (size_t)stage_bytes * p.stages + 1024 + 24 * p.stages + 64;
+    const size_t smem = (size_t)stage_bytes * p.stages + 1024 + 24 * p.stages + 80;
     if (smem > (size_t)SMEM_ATTR) return -6;
     const long long tiles = (long long)((g.M + TM - 1) / TM) * ((g.N + p.bn - 1) / p.bn) * g.batch * p.ksplit;
     if (tiles > (1ll << 30)) return -4;
     int grid = (int)(tiles < sms ? tiles : sms);
     if (g.grid_cap > 0 && grid > g.grid_cap) grid = g.grid_cap;
     if (g.prec == PPL_PREC_BF16X3)
-        launch_tc<PPL_PREC_BF16X3>(drain, grid, smem, s, a);
+        launch_tc<PPL_PREC_BF16X3>(mode, grid, smem, s, a);
     else if (g.prec == PPL_PREC_TF32X3)
-        launch_tc<PPL_PREC_TF32X3>(drain, grid, smem, s, a);
+        launch_tc<PPL_PREC_TF32X3>(mode, grid, smem, s, a);
     else
-        launch_tc<PPL_PREC_TF32>(drain, grid, smem, s, a);
+        launch_tc<PPL_PREC_TF32>(mode, grid, smem, s, a);
     const cudaError_t le = cudaGetLastError();
     return le == cudaSuccess ? 0 : -(1000 + (int)le);
 }
@@ -1168,7 +1351,7 @@ struct GroupNode {
 }  // namespace
 
 const void* tc_group_kernel(const void* f) {
-    for (int i = 0; i < 6; ++i)
+    for (int i = 0; i < NKERN; ++i)
         if (k_single[i] == f) return k_grouped[i];
     return nullptr;
 }
@@ -1178,7 +1361,7 @@ int tc_group_capacity() { return TC_GROUP_MAX; }
 int tc_group_node_params(const void* f, const void* const* args, int n, cudaKernelNodeParams* out, void** storage) {
     *storage = nullptr;
     int ki = -1;
-    for (int i = 0; i < 6; ++i)
+    for (int i = 0; i < NKERN; ++i)
         if (k_single[i] == f) ki = i;
     if (ki < 0 || n < 1 || n > TC_GROUP_MAX || !args || !out) return -1;
     if (tc_init_driver() != 0) return -1;
@@ -1209,11 +1392,11 @@ int tc_group_node_params(const void* f, const void* const* args, int n, cudaKern
         return -4;
     }
     a.tile0[n] = (int)tot;
-    const int planes = (ki / 2 == 1) ? 1 : 2;   // TF32 one plane; BF16X3 and TF32X3 hi and lo
+    const int planes = (ki / 3 == 1) ? 1 : 2;   // TF32 one plane; BF16X3 and TF32X3 hi and lo
     const int stage_bytes = planes * (TM + a.bn_max) * KROW_BYTES;
     a.stages = SMEM_BUDGET / stage_bytes;
     if (a.stages > 8) a.stages = 8;
-    const size_t smem = (size_t)stage_bytes * a.stages + 1024 + 24 * a.stages + 64;
+    const size_t smem = (size_t)stage_bytes * a.stages + 1024 + 24 * a.stages + 80;
     if (a.stages < 2 || smem > (size_t)SMEM_ATTR) {
         delete g;
         return -6;
@@ -1222,7 +1405,7 @@ int tc_group_node_params(const void* f, const void* const* args, int n, cudaKern
     *out = cudaKernelNodeParams{};
     out->func = const_cast<void*>(k_grouped[ki]);
     out->gridDim = dim3((unsigned)(tot < sms ? tot : sms));
-    out->blockDim = dim3(NTHREADS);
+    out->blockDim = dim3((unsigned)threads_of(ki % 3));
     out->sharedMemBytes = (unsigned)smem;
     out->kernelParams = g->params;
     out->extra = nullptr;

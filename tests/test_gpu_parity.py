@@ -143,6 +143,31 @@ def test_restarted_accumulation_mttkrp(prec, chunk, steps, shape):
     cp.close()
 
 
+@pytest.mark.parametrize("prec", ["bf16x3", "tf32", "tf32x3"])
+@pytest.mark.parametrize("shape", [(2, 33, 159, 161),   # two K blocks; tiles just below and above 160 columns
+                                   (3, 64, 17, 7),      # whole K blocks, one narrow tile
+                                   (2, 256, 161, 320),  # eight full K blocks, the most handed over (32-wide)
+                                   (2, 257, 33, 48)])   # one more: the wide tiles
+def test_short_restarted_sums_handed_over(prec, shape):
+    """Restarted accumulation at the edges of the form that hands finished tiles to
+    storing warps: number of K blocks, tile width, column and row remainders.  The
+    element-wise chain bound and the normwise one hold for every mode; the per-column
+    one is for columns of many rows (with o = 2 a column's largest entry can itself
+    be a small one)."""
+    o, v, X, R = shape
+    inp = inputs.make_inputs(o, v, X, R, seed=3)
+    refs, abss = _mttkrp_refs(inp.Bvv, inp.tau, inp.factors)
+    cp = binding.CpAls(_dev(inp.B), _dev(inp.tau), inp.factors, precision=prec, acc_chunk=1)
+    for m in orc.MODES:
+        M = cp.mttkrp(m).cpu().numpy()
+        what = f"{prec} {shape} mode {m}"
+        check_abs_bound(M, refs[m], abss[m], GAMMA[prec], what)
+        if len(refs[m]) > 4:
+            check_columns(M, refs[m], COLTOL[prec], what)
+        assert _rel(M, refs[m]) < TOL_MTTKRP[prec]
+    cp.close()
+
+
 @pytest.mark.parametrize("shape", SHAPES)
 def test_fp64_sweeps_match_oracle(shape):
     o, v, X, R = shape
