@@ -652,7 +652,7 @@ int run_tc_partial(ppl_cpd* h, TcGemm& g, double* out, long long ldo, const char
     g.out.ns = g.M;
     int e = run_tc(h, g, what);
     if (e) return e;
-    reduce_partials(part, ks, g.M, g.N, out, ldo, h->st);
+    reduce_partials(part, g.out.sk, 0, ks, g.M, g.N, 1, out, ldo, 0, h->st);
     return PPL_OK;
 }
 

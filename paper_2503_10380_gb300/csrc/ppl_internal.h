@@ -150,8 +150,10 @@ struct TcGemm {
     TcOut out;
 };
 int tc_gemm(const TcGemm& g, unsigned int* err_flag, cudaStream_t s);
-// out[m * ldo + n] = sum_k part[k][n][m] (FP64 sum of FP32 split-K partials, deterministic)
-void reduce_partials(const float* part, int ksplit, int M, int N, double* out, long long ldo, cudaStream_t s);
+// out[z * ob + m * ldo + n] = sum_k part[k * sk + z * sb + n * M + m] (FP64 sum of FP32
+// split-K partials in the order of k)
+void reduce_partials(const float* part, long long sk, long long sb, int ksplit, int M, int N, int batch, double* out,
+                     long long ldo, long long ob, cudaStream_t s);
 // dst[b][j][i] = src[b][i][j], i, j < n, operand planes of the given precision
 void transpose_operand(int prec, const void* src, void* dst, long long plane_elems, int n, long long ld,
                        long long bstride, int batch, cudaStream_t s);

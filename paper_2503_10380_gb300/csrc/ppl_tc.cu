@@ -846,16 +846,52 @@ const void* const k_grouped[NKERN] = {
     (const void*)k_tc_gemm_group<PPL_PREC_TF32X3, 0>, (const void*)k_tc_gemm_group<PPL_PREC_TF32X3, 1>,
     (const void*)k_tc_gemm_group<PPL_PREC_TF32X3, 2>};
 
-// Sum split-K partials part[ks][n][m] (fp32) in FP64 into out[m * ldo + n].
-__global__ void k_reduce_partials(const float* part, int ksplit, int M, int N, double* out, long long ldo) {
-    const long long total = (long long)M * N;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int m = (int)(e % M), n = (int)(e / M);
-        double s = 0.0;
-        for (int k = 0; k < ksplit; ++k) s += (double)part[(long long)k * total + e];
-        out[(long long)m * ldo + n] = s;
+// Sum split-K partials part[ks][n][m] (fp32) in FP64, in the order of the slices, into
+// out[m * ldo + n], with strides between the slices and between the entries of a batch
+// (blockIdx.y).  One thread per element, RPU slices in registers while the next RPU are
+// on their way.  An FP64 instruction occupies an SM sub-partition for 64 clocks, and a
+// conversion as much as an addition, so the operands are widened by integer instructions
+// (a normal number's exponent rebiased; a zero is the double zero); RPU slices with
+// a subnormal, an infinity or a NaN among them are converted.  With one conversion and one
+// load at a time per slice before: 200 x 800 elements of 19 slices 15.7 -> 9.8 us,
+// 117 x 331 of 76 13.6 -> 9.8, 48 x 400 of 76 15.7 -> 6.8, eight uneven instances' 48
+// reductions 3.2 -> 1.3 ms.
+constexpr int RPU = 16, RPT = 128;
+__global__ void __launch_bounds__(RPT) k_reduce_partials(const float* part, long long sk, long long sb, int ksplit, int M,
+                                                         int N, double* out, long long ldo, long long ob) {
+    const long long e = (long long)blockIdx.x * RPT + threadIdx.x;
+    if (e >= (long long)M * N) return;
+    const float* x = part + (long long)blockIdx.y * sb + e;
+    double s = 0.0;
+    unsigned nxt[RPU];
+#pragma unroll
+    for (int u = 0; u < RPU; ++u) nxt[u] = u < ksplit ? __float_as_uint(__ldg(x + u * sk)) : 0u;
+#pragma unroll 1
+    for (int k = 0; k < ksplit; k += RPU) {
+        unsigned cur[RPU];
+        bool normal = true;
+#pragma unroll
+        for (int u = 0; u < RPU; ++u) {
+            cur[u] = nxt[u];
+            normal &= ((cur[u] << 1) - 0x1000000u < 0xfe000000u) || (cur[u] << 1) == 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < RPU; ++u) nxt[u] = k + RPU + u < ksplit ? __float_as_uint(__ldg(x + (k + RPU + u) * sk)) : 0u;
+        if (normal) {
+#pragma unroll
+            for (int u = 0; u < RPU; ++u) {
+                if (k + u < ksplit) {
+                    const unsigned b = cur[u], h = (b << 1) ? ((b & 0x7fffffffu) >> 3) + (896u << 20) : 0u;
+                    s += __hiloint2double((int)((b & 0x80000000u) | h), (int)(b << 29));
+                }
+            }
+        } else {
+#pragma unroll 1
+            for (int u = 0; u < RPU && k + u < ksplit; ++u) s += (double)__ldg(x + (k + u) * sk);
+        }
     }
+    const int m = (int)(e % M), n = (int)(e / M);
+    out[(long long)blockIdx.y * ob + (long long)m * ldo + n] = s;
 }
 
 // Batched transpose of operand planes: dst[b][j][i] = src[b][i][j] for i, j < n
@@ -1260,10 +1296,11 @@ int tc_gemm(const TcGemm& g, unsigned int* err_flag, cudaStream_t s) {
     return le == cudaSuccess ? 0 : -(1000 + (int)le);
 }
 
-void reduce_partials(const float* part, int ksplit, int M, int N, double* out, long long ldo, cudaStream_t s) {
-    const long long total = (long long)M * N;
-    if (total <= 0) return;
-    k_reduce_partials<<<grid_for(total, 256), 256, 0, s>>>(part, ksplit, M, N, out, ldo);
+void reduce_partials(const float* part, long long sk, long long sb, int ksplit, int M, int N, int batch, double* out,
+                     long long ldo, long long ob, cudaStream_t s) {
+    if (M <= 0 || N <= 0 || batch <= 0) return;
+    const long long blocks = ((long long)M * N + RPT - 1) / RPT;
+    k_reduce_partials<<<dim3((unsigned)blocks, (unsigned)batch), RPT, 0, s>>>(part, sk, sb, ksplit, M, N, out, ldo, ob);
 }
 
 void transpose_operand(int prec, const void* src, void* dst, long long plane_elems, int n, long long ld,

@@ -168,6 +168,25 @@ def test_short_restarted_sums_handed_over(prec, shape):
     cp.close()
 
 
+@pytest.mark.parametrize("spread", [0, 12, 40, 80])
+@pytest.mark.parametrize("shape", [(5, 24, 72, 48), (3, 33, 97, 9)])
+def test_split_k_slices_of_mixed_magnitude(shape, spread):
+    """Split-K slices whose exponents lie up to 2 spread apart: the sum over slices as
+    integers, the FP64 loop beyond its range, and elements on both sides of it in one
+    tile.  Column r of the result has its own scale, so the chain bound and the
+    per-column bound hold as they do without the scaling."""
+    o, v, X, R = shape
+    inp = inputs.make_inputs(o, v, X, R, seed=4)
+    scale = 2.0 ** np.round(np.linspace(-spread / 2, spread / 2, X))
+    B = inp.B * np.random.default_rng(4).permutation(scale)[:, None, None]
+    refs, abss = _mttkrp_refs(B[:, o:, o:], inp.tau, inp.factors)
+    cp = binding.CpAls(_dev(B), _dev(inp.tau), inp.factors, precision="tf32x3")
+    for m in orc.MODES:
+        M = cp.mttkrp(m).cpu().numpy()
+        check_mttkrp(M, refs[m], abss[m], "tf32x3", f"{shape} spread {spread} mode {m}")
+    cp.close()
+
+
 @pytest.mark.parametrize("shape", SHAPES)
 def test_fp64_sweeps_match_oracle(shape):
     o, v, X, R = shape
