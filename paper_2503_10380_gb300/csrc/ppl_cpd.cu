@@ -46,7 +46,7 @@ struct Layout {
     long long nrowx;
     int rcr;
     size_t total;
-    int rc, na;
+    int rc, na, ng;               // r-chunk; rows a per launch of the exact contraction, FP64 and tensor-core
     long long ldv, ldX, ldo2, ldvv;
     long long ldk;   // tensor-core form: v padded to the K-panel width (a K extent of v per block of a compound index)
     int ke;          // the K-panel width: elements of one 128-byte operand row
@@ -54,6 +54,10 @@ struct Layout {
 
 constexpr int NPART = 2 * 304 + 8;
 constexpr int KSMAX = 80;   // most split-K slices of one tensor-core contraction
+// Bound of G of the rows a that one launch of the tensor-core exact contraction takes (the
+// FP64 form's block of G, in which the partials of the mixed form lie, is as large).
+// At o 20, v 120, X 360: 64 MB 3.63 ms, 128 MB 2.83, 256 MB 2.42, one row per launch 7.29.
+constexpr size_t EXACT_BYTES = (size_t)256 << 20;
 constexpr int RC_MAX = 1024; // most rank columns per pass of the chain
 #ifndef TF32X3_ACC_STEPS
 #define TF32X3_ACC_STEPS 0      // default MMA K steps per TF32X3 accumulation chunk (0: a K block)
@@ -163,6 +167,7 @@ bool plan(int o, int v, int X, int R, const ppl_cpd_opts& op, Layout& L) {
     L.PART = none;
     L.Bbar = L.BbN = L.BbP = L.BbT = none;
     L.Bq = L.BbQ = L.Gop = none;
+    L.ng = 0;
     if (op.dressed) L.Bbar = take((size_t)X * v * v * d);
     if (!tc) {
         L.T64 = take((size_t)R * v * v * d);
@@ -194,11 +199,19 @@ bool plan(int o, int v, int X, int R, const ppl_cpd_opts& op, Layout& L) {
         L.S = take((size_t)rc * kvv * e);                  // rows r, K = (c, d)
         {
             const size_t chain_part = (size_t)KSMAX * (size_t)(v > o * o ? v : o * o) * rc;
-            const size_t exact_part = (size_t)KSMAX * (size_t)v * o * o;
+            // rows a of the exact contraction per launch: their G within EXACT_BYTES, the
+            // split-K partials of more than one within the FP64 form's block of G
+            const size_t part1 = (size_t)KSMAX * (size_t)v * o * o * sizeof(float);
+            long long ng = (long long)(EXACT_BYTES / ((size_t)v * kvv * e));
+            const long long np = (long long)((size_t)na * v3 * d / part1);
+            if (ng > np) ng = np;
+            if (ng > na) ng = na;
+            L.ng = ng < 1 ? 1 : (int)ng;
+            const size_t exact_part = part1 / sizeof(float);
             L.PART = take((chain_part > exact_part ? chain_part : exact_part) * sizeof(float));
         }
         L.Bq = take(vv * kX * e);                          // rows (p,q), K = Q
-        L.Gop = take((size_t)v * kvv * e);                 // rows b, K = (c, d)
+        L.Gop = take((size_t)L.ng * v * kvv * e);          // per a: rows b, K = (c, d)
         if (op.dressed) L.BbQ = take(vv * kX * e);
         if (op.dressed) {
             L.BbN = take(Xv * L.ldk * e);
@@ -633,9 +646,9 @@ int t_tc(ppl_cpd* h) {
     return PPL_OK;
 }
 
-// split-K contraction through FP32 partials [ks][n][m] in L.PART, then an FP64
-// reduction into out[m * ldo + n]
-int run_tc_partial(ppl_cpd* h, TcGemm& g, double* out, long long ldo, const char* what) {
+// split-K contraction through FP32 partials part[batch][ks][n][m], then an FP64
+// reduction into out[z * ob + m * ldo + n]
+int run_tc_partial(ppl_cpd* h, TcGemm& g, float* part, double* out, long long ldo, long long ob, const char* what) {
     g.prec = h->opts.precision;
     if (g.bn == 0) g.bn = bn_for(g.N);
     g.ksplit = auto_ksplit(g.M, g.N, g.bn, g.K, g.prec);
@@ -643,16 +656,16 @@ int run_tc_partial(ppl_cpd* h, TcGemm& g, double* out, long long ldo, const char
     const int nkb = (g.K + ke - 1) / ke;
     const int per = (nkb + g.ksplit - 1) / g.ksplit;
     const int ks = (nkb + per - 1) / per;      // the split count the kernel will use
-    float* part = h->at<float>(h->L.PART);
     g.out = TcOut{};
     g.out.kind = EPI_F32;
     g.out.out = part;
     g.out.sk = (long long)g.M * g.N;
+    g.out.sb = g.out.sk * ks;
     g.out.q0p = ke; g.out.q0s = 1;
     g.out.ns = g.M;
     int e = run_tc(h, g, what);
     if (e) return e;
-    reduce_partials(part, g.out.sk, 0, ks, g.M, g.N, 1, out, ldo, 0, h->st);
+    reduce_partials(part, g.out.sk, g.out.sb, ks, g.M, g.N, g.batch, out, ldo, ob, h->st);
     return PPL_OK;
 }
 
@@ -702,7 +715,7 @@ int chain_tc(ppl_cpd* h, int mode, double* Mout, bool keep_wa) {
         g3.A = pmat(opb(h, (mode == 1 && h->dressed()) ? h->L.BbP : h->L.Bp), pBn, v, KY, 1, v, 0);
         g3.B = pmat(opb(h, h->L.Y), pW, rcur, KY, 1, rc, 0);
         g3.M = v; g3.N = rcur; g3.K = KY; g3.batch = 1;
-        e = run_tc_partial(h, g3, Mout + r0, R, "M");
+        e = run_tc_partial(h, g3, h->at<float>(h->L.PART), Mout + r0, R, 0, "M");
         if (e) return e;
     }
     return PPL_OK;
@@ -761,7 +774,7 @@ int p_tc_body(ppl_cpd* h, bool wa_ready) {
         gp.A = pmat(opb(h, h->L.tauN), (long long)o * o * q.kvv, o * o, (int)q.kvv, 1, (long long)o * o, 0);
         gp.B = pmat(opb(h, h->L.S), pS, rcur, (int)q.kvv, 1, rc, 0);
         gp.M = o * o; gp.N = rcur; gp.K = (int)q.kvv; gp.batch = 1;
-        e = run_tc_partial(h, gp, P + r0, R, "P");
+        e = run_tc_partial(h, gp, h->at<float>(h->L.PART), P + r0, R, 0, "P");
         if (e) return e;
     }
     return PPL_OK;
@@ -852,7 +865,7 @@ int prepare_operands(ppl_cpd* h, bool tau_only) {
     zero_bytes(opb(h, h->L.WTa), (size_t)h->R * v * q.kX * eb, h->st);
     zero_bytes(opb(h, h->L.WTb), (size_t)h->L.rc * v * q.kX * eb, h->st);
     zero_bytes(opb(h, h->L.S), (size_t)h->L.rc * q.kvv * eb, h->st);
-    zero_bytes(opb(h, h->L.Gop), (size_t)v * q.kvv * eb, h->st);
+    zero_bytes(opb(h, h->L.Gop), (size_t)h->L.ng * v * q.kvv * eb, h->st);
     return PPL_OK;
 }
 
@@ -1351,14 +1364,19 @@ int ppl_exact_contract_mixed(ppl_cpd* h, double* normR2, double* E_exact, double
     g.M = o * v; g.N = o * v; g.K = X; g.batch = 1; g.ksplit = 1; g.alpha = 1.0;
     gemm(h, g);
     const Pan pq = pan_of(h);
-    const long long pQ = (long long)v * v * pq.kX, pG = (long long)v * pq.kvv;
-    for (int a = 0; a < v && !e; ++a) {
-        // G_a[b][c][d] = sum_Q D-bar[Q][b][d] B[Q][a][c]; stored rows b, K (c, d): m = b*v + d, n = c
+    // ng rows a per launch: one row's five launches of 5 to 17 us each ended in a tail of
+    // idle SMs and a gap
+    const int ng = h->L.ng;
+    const long long pQ = (long long)v * v * pq.kX, bG = (long long)v * pq.kvv, pG = bG * ng;
+    float* part = h->at<float>(ng > 1 ? h->L.Gblk : h->L.PART);
+    for (int a = 0; a < v && !e; a += ng) {
+        const int nb = (v - a < ng) ? v - a : ng;
+        // G_a[b][c][d] = sum_Q D-bar[Q][b][d] B[Q][a][c]; per a: rows b, K (c, d); m = b*v + d, n = (a, c)
         TcGemm g1{};
         g1.A = pmat(opb(h, h->dressed() ? h->L.BbQ : h->L.Bq), pQ, v * v, X, 1, (long long)v * v, 0);
         g1.B = pmat(opb(h, h->L.Bq), pQ, v * v, X, 1, (long long)v * v, 0);
         g1.b_row0 = a * v;
-        g1.M = v * v; g1.N = v; g1.K = X; g1.batch = 1; g1.ksplit = 1;
+        g1.M = v * v; g1.N = nb * v; g1.K = X; g1.batch = 1; g1.ksplit = 1;
         g1.out = out_map(opb(h, h->L.Gop), pG, 0, v, plain(pq.ke, pq.ke), kpan((long long)v * pq.ke),
                          pq.ldk * v);
         e = run_tc(h, g1, "exact G");
@@ -1366,12 +1384,13 @@ int ppl_exact_contract_mixed(ppl_cpd* h, double* normR2, double* E_exact, double
         // R[a][b][ij] = sum_{cd} G_a[b][cd] tau[ij][cd], split-K summed in FP64
         double* Rdst = R_out ? R_out + (long long)a * vo2 : h->at<double>(h->L.Rblk);
         TcGemm g2{};
-        g2.A = pmat(opb(h, h->L.Gop), pG, v, (int)pq.kvv, 1, v, 0);
+        g2.A = pmat(opb(h, h->L.Gop), pG, v, (int)pq.kvv, nb, v, bG);
+        g2.a_bstep = 1;
         g2.B = pmat(opb(h, h->L.tauN), (long long)o * o * pq.kvv, o * o, (int)pq.kvv, 1, (long long)o * o, 0);
-        g2.M = v; g2.N = o * o; g2.K = (int)pq.kvv; g2.batch = 1;
-        e = run_tc_partial(h, g2, Rdst, (long long)o * o, "exact R");
+        g2.M = v; g2.N = o * o; g2.K = (int)pq.kvv; g2.batch = nb;
+        e = run_tc_partial(h, g2, part, Rdst, (long long)o * o, vo2, "exact R");
         if (e) break;
-        exact_reduce(Rdst, a, 1, v, o, gov, h->at<double>(h->L.partial), acc, h->st);
+        exact_reduce(Rdst, a, nb, v, o, gov, h->at<double>(h->L.partial), acc, h->st);
     }
     if (!e) e = check_cuda(h, "exact_contract_mixed");
     if (!e) e = sync_and_check(h);

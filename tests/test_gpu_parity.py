@@ -587,6 +587,25 @@ def test_exact_contraction_on_tensor_cores(prec, tol, dressed):
     cp.close()
 
 
+@pytest.mark.parametrize("prec", ["bf16x3", "tf32x3"])     # 36 and 27 rows a per launch: remainders 25 and 16
+def test_exact_contraction_on_tensor_cores_in_groups(prec):
+    """Several rows a per launch, the last group smaller: R into the caller's tensor and,
+    without one, only the sums (the same ones)."""
+    inp = inputs.make_inputs(8, 97, 41, 20, seed=45)
+    cp = binding.CpAls(_dev(inp.B), _dev(inp.tau), inp.factors, precision=prec)
+    n2, E, Rt = cp.exact_contract(want_R=True, mixed=True)
+    assert cp.exact_contract(mixed=True)[:2] == (n2, E)
+    R_ref = orc.ppl_tensor(inp.Bvv, inp.tau)
+    R_abs = orc.ppl_tensor(np.abs(inp.Bvv), np.abs(inp.tau))
+    Rg = Rt.cpu().numpy()
+    o, v = inp.o, inp.Bvv.shape[1]
+    check_abs_bound(Rg, R_ref, R_abs, GAMMA[prec], f"{prec} R in groups")
+    check_columns(Rg.reshape(v * v, o * o), R_ref.reshape(v * v, o * o), COLTOL[prec], f"{prec} R per (i,j)")
+    assert abs(n2 - float(np.sum(Rg ** 2))) <= 1e-12 * n2
+    assert abs(E - orc.energy_of_tensor(Rg, inp.B, o)) <= 1e-10 * abs(E)
+    cp.close()
+
+
 def test_full_size_benchmark_instance():
     """o=20 v=200 X=600 R=800, the benchmark's instance, in the configuration bench.py
     times (graph replay, r-chunk from the autotuner): every MTTKRP against the oracle,
