@@ -56,7 +56,7 @@ constexpr int NPART = 2 * 304 + 8;
 constexpr int KSMAX = 80;   // most split-K slices of one tensor-core contraction
 // Bound of G of the rows a that one launch of the tensor-core exact contraction takes (the
 // FP64 form's block of G, in which the partials of the mixed form lie, is as large).
-// At o 20, v 120, X 360: 64 MB 3.63 ms, 128 MB 2.83, 256 MB 2.42, one row per launch 7.29.
+// At o 14, v 120, X 360: 64 MB 3.63 ms, 128 MB 2.83, 256 MB 2.42, one row per launch 7.29.
 constexpr size_t EXACT_BYTES = (size_t)256 << 20;
 constexpr int RC_MAX = 1024; // most rank columns per pass of the chain
 #ifndef TF32X3_ACC_STEPS

@@ -493,6 +493,33 @@ def test_batch_of_uneven_instances_equals_individual_sweeps():
         p.close()
 
 
+@pytest.mark.parametrize("shapes", [
+    [(3, 20, 40, 1)] * 9 + [(6, 90, 200, 330)],           # one large among the smallest: two blocks each
+    [(4, 33, 66, 97)] * 5,                                # equal ones
+    [(6, 17, 30, 33 + 16 * k) for k in range(24)],        # many, of every number of block steps (R < v o^2)
+    [(5, 50, 100, 150)],                                  # one alone
+])
+def test_batched_solves_share_the_blocks(shapes):
+    """The blocks that an instance of a batch gets depend on the others; its factors do
+    not.  The solve of one instance forms every sum in the same order on any number of
+    blocks, so the tolerance is that of the last bits (FP64 handles: no operand
+    rounding lies between)."""
+    inps = [inputs.make_inputs(*sh, seed=60 + k) for k, sh in enumerate(shapes)]
+    probs = [binding.CpAls(_dev(i.B), _dev(i.tau), i.factors, precision="fp64") for i in inps]
+    batch = binding.Batch(probs, nstreams=4)
+    batch.sweep(1)
+    for k, (p, i) in enumerate(zip(probs, inps)):
+        q = binding.CpAls(_dev(i.B), _dev(i.tau), i.factors, precision="fp64")
+        q.sweep(1)
+        fp, fq = _factors(p), _factors(q)
+        for m in fp:
+            check_columns(fp[m].reshape(-1, fp[m].shape[-1]), fq[m].reshape(-1, fq[m].shape[-1]), 1e-9, f"instance {k} {m}")
+        q.close()
+    batch.close()
+    for p in probs:
+        p.close()
+
+
 @pytest.mark.parametrize("prec,tol", [("fp64", 1e-8), ("tf32x3", 2e-4)])
 def test_batch_of_uneven_instances_against_oracle(prec, tol):
     """Four uneven instances swept together from one graph (each on its share of
