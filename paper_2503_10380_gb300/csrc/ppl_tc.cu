@@ -21,7 +21,8 @@
 // 0 issues TMA into a ring of shared-memory stages, lane 0 of warp 1 issues the
 // MMAs into one of two TMEM accumulators, and eight warps drain the other
 // accumulator to global memory, so a tile's epilogue overlaps the next tile's
-// mainloop.  Warp 2 owns the TMEM allocation.
+// mainloop; with restarted sums over a short K four more warps do the writing (the
+// handed-over form below).  Warp 2 owns the TMEM allocation.
 // Every mbarrier wait is bounded; on expiry the kernel records the error,
 // drains what it issued, frees TMEM and returns.
 #include "ppl_internal.h"
@@ -50,11 +51,11 @@ constexpr unsigned long long WAIT_NS = 500ull * 1000ull * 1000ull;   // 0.5 s pe
 // lanes of its quarter, warp % 4), each draining one 128-column half of the tile
 // as four 32-column pieces.  With the accumulator restarted every K block an
 // epilogue thread holds 128 running sums and 64 columns in flight from TMEM (the
-// next piece's load under the current one's additions), more registers than a 384-thread block gives every thread, so the
-// control warpgroup hands registers to the epilogue (setmaxnreg): 56 for it and
-// 224 for each epilogue thread, 128*56 + 256*224 = 384*168, exactly the launch's
-// allocation (checked on the host before every launch: a split above the
-// allocation would wait forever).
+// next piece's load under the current one's additions), more registers than a 384-thread
+// block gives every thread, so the control warpgroup hands registers to the epilogue
+// (setmaxnreg): 56 for it and 224 for each epilogue thread, 128*56 + 256*224 = 384*168,
+// exactly the launch's allocation (checked on the host before every launch: a split
+// above the allocation would wait forever).
 constexpr int NCTRL = 4;                      // warps of the control warpgroup
 constexpr int NEPI = 8;                       // epilogue warps
 constexpr int NTHREADS = 32 * (NCTRL + NEPI);
@@ -854,7 +855,7 @@ const void* const k_grouped[NKERN] = {
 // (a normal number's exponent rebiased; a zero is the double zero); RPU slices with
 // a subnormal, an infinity or a NaN among them are converted.  With one conversion and one
 // load at a time per slice before: 200 x 800 elements of 19 slices 15.7 -> 9.8 us,
-// 117 x 331 of 76 13.6 -> 9.8, 48 x 400 of 76 15.7 -> 6.8, eight uneven instances' 48
+// 117 x 331 of 75 13.6 -> 9.8, 90 x 96 of 74 15.7 -> 6.8, sixteen uneven instances' 48
 // reductions 3.2 -> 1.3 ms.
 constexpr int RPU = 16, RPT = 128;
 __global__ void __launch_bounds__(RPT) k_reduce_partials(const float* part, long long sk, long long sb, int ksplit, int M,
