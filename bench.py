@@ -39,7 +39,7 @@ MAIN_CFG = (60, 600, 1800, 2400)   # the largest single-GPU configuration (o, v,
 CFG1 = (20, 200, 600, 800)
 CFG2 = (40, 400, 1200, 1600)
 O, V, XAUX, RANK = CFG1            # the instance the oracle's flop rate is timed on for estimates
-ACC_SWEEPS_MAIN = 2                # sweeps compared against the FP64 GPU form (about 37 s per FP64 sweep)
+ACC_SWEEPS_MAIN = 2                # sweeps compared against the FP64 GPU form (about 3 s per FP64 sweep)
 E2E_SWEEPS, E2E_STEPS = 10, 2
 def _workload(cfg):
     return f"cp-als-ppl single instance o={cfg[0]} v={cfg[1]} X={cfg[2]} R={cfg[3]}, graph-replayed ALS sweeps"
