@@ -796,7 +796,7 @@ struct SolveBatch {
     SolveP p[MAX_BATCH];
 };
 
-__global__ void __launch_bounds__(NT, 2) k_solve_batch(const __grid_constant__ SolveBatch b) {
+__global__ void __launch_bounds__(NT, 3) k_solve_batch(const __grid_constant__ SolveBatch b) {
     int l = 0;
     while (l + 1 < b.nl && b.lane_blk0[l + 1] <= (int)blockIdx.x) ++l;
     const int bid = (int)blockIdx.x - b.lane_blk0[l], G = b.lane_blk0[l + 1] - b.lane_blk0[l];
@@ -915,14 +915,16 @@ int solve_modes_batched(const SolveArgs* a, int n, cudaStream_t s) {
             cudaGetLastError();
             return -2;
         }
-        // two blocks per SM: a third one's FP64 instructions stretch the factorisations of
-        // the others' diagonal blocks by more than it brings (6.51 -> 6.00 ms with three
-        // and 5.44 with two, six instances)
-        g_batch_per_sm = per > 2 ? 2 : per;
+        g_batch_per_sm = per;
     }
-    const int cap = g_batch_per_sm * sms;   // blocks that are co-resident in one cooperative launch
     for (int k0 = 0; k0 < n; k0 += MAX_BATCH) {
         const int nb = (n - k0 < MAX_BATCH) ? n - k0 : MAX_BATCH;
+        // Two blocks per SM for few instances: a third one's FP64 instructions stretch the
+        // factorisations of the others' diagonal blocks by more than it brings (sweeps of 6
+        // instances 6.00 ms with three and 5.44 with two, 16 instances 27.97 and 27.69; but
+        // 24 instances 38.4 and 43.1, 64 79.1 and 81.9)
+        const int per_sm = nb <= 16 && g_batch_per_sm > 2 ? 2 : g_batch_per_sm;
+        const int cap = per_sm * sms;   // blocks that are co-resident in one cooperative launch
         if (2 * nb > cap) return -3;
         SolveBatch b;
         b.n = nb;
@@ -940,7 +942,7 @@ int solve_modes_batched(const SolveArgs* a, int n, cudaStream_t s) {
         // FP64 work at G blocks' share of the FP64 rate (2 FMA per clock per SM at
         // about 2 GHz, shared by the blocks of an SM) plus a latency per 32-wide
         // block step; L is the one with the shortest modelled makespan.
-        const double rate_blk = 8.0e9 / g_batch_per_sm, step_s = 20e-6;
+        const double rate_blk = 8.0e9 / per_sm, step_s = 20e-6;
         auto est = [&](int k, int G) { return work[k] / ((double)(G < want[k] ? G : want[k]) * rate_blk) + steps[k] * step_s; };
         int best_L = 0, best_lane[MAX_BATCH] = {};
         double best_span = 0.0;
@@ -974,11 +976,12 @@ int solve_modes_batched(const SolveArgs* a, int n, cudaStream_t s) {
         // Or every instance in a lane of its own, with as many blocks as its work needs to
         // finish at the same time T as the others: the shortest such T, by bisection.
         // Equal lanes leave the SMs of the small instances idle while the largest one
-        // ends.  Sweeps of uneven batches, this and two blocks per SM: 16 instances of
-        // v 50 .. 234 29.2 -> 27.7 ms, four to eight instances 10 to 20 per cent less.
+        // ends.  Sweeps of uneven batches: 16 instances of v 50 .. 234 29.2 -> 27.7 ms, 24
+        // 40.3 -> 38.4, four to eight instances 10 to 20 per cent less.
         int own[MAX_BATCH];
         const double own_span = own_lanes(nb, cap, want, work, steps, rate_blk, step_s, own);
-        const bool use_own = own_span > 0.0 && own_span < best_span;
+        // (not below 14 blocks each: 40 instances 59.7 ms against 57.5 in equal lanes)
+        const bool use_own = own_span > 0.0 && own_span < best_span && cap >= 14 * nb;
         if (use_own) best_L = nb;
         b.nl = best_L;
         int blk = 0, q = 0;
