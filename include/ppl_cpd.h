@@ -46,7 +46,11 @@ extern "C" {
 #define PPL_ENOTREADY 5   /* fit asked for before ||R||^2 or before any sweep       */
 
 /* arithmetic of the MTTKRP contractions; Gram, solve, fit and energy are FP64 always */
-#define PPL_PREC_FP64   0  /* plain FP64 on the CUDA cores                                 */
+#define PPL_PREC_FP64   0  /* FP64: contractions of K >= 8 by exact digit products on the
+                              tensor cores (sums in 64-bit fixed point below the rows'
+                              largest entries, rounded to FP64 once; elements for which that
+                              would be less accurate than FP64 FMAs are formed by FMAs),
+                              the others with FP64 FMAs                                    */
 #define PPL_PREC_BF16X3 1  /* tcgen05 BF16 hi/lo split, hi*hi + hi*lo + lo*hi, FP32 accum. */
 #define PPL_PREC_TF32   2  /* tcgen05 TF32 (round-to-nearest operands), FP32 accumulate    */
 #define PPL_PREC_TF32X3 3  /* tcgen05 TF32 hi/lo split (22 bits), three products, FP32

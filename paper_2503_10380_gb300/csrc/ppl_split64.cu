@@ -4,34 +4,38 @@
 // GB300 executes two FP64 FMAs per clock per SM (1.25 TFLOP/s in all), so every
 // FP64 contraction of the library was bound by that pipe.  Here each row of A and
 // each row of B (column of the product) is scaled by the power of two above its
-// largest entry and written as a 56-bit fixed-point number in seven balanced
+// largest entry and written as a 64-bit fixed-point number in eight balanced
 // base-256 digits (after Ozaki, Ogita, Oishi & Rump, "Error-free transformations of
 // matrix multiplication", Numer. Algorithms 59, 2012; for matrix units, Mukunoki et
 // al., ISC 2020).  A digit with its weight, d 256^-i, is exact in bf16, a product of
 // two is d d' 256^-(i+j) with |d d'| <= 2^14, and up to 7 x 128 products of one weight
 // add up below 2^24 units, so tcgen05.mma with its FP32 accumulator forms those sums
 // without rounding.  There are seven accumulators, for the weights 0 .. 6; the last also
-// takes the products of weight 7 (where its rounding is below the unit of the
+// takes the products of weight 7, the least kept (its rounding is below the unit of the
 // result's last digit).  Every 128 values of k they are folded into an integer
 // accumulator of 88 bits, and the result is rounded to FP64 once.
 //
-// Error: the fixed-point rounding of the entries, 2^-56 of the row's power of two
-// each, and the products of weight 8 and above, 2^-64.  Where all of a row's entries
-// matter about equally this is below the rounding of an FP64 sum.  An element whose
-// terms are all small against its row maxima would lose relative accuracy: an eighth
-// accumulator sums the products of the leading digits' absolute values, and if that
-// sum is below half the sum of the two rows' norms (in units of the leading digit) the
-// element's error could exceed 2^-48 of the sum of its |terms| (K = 32 roundings of an
-// FP64 sum).  Then the block computes its tile with FP64 FMAs instead, as it does for a
-// row with an Inf, a NaN or only entries below 2^-959.
+// Error: the fixed-point rounding of the entries, 2^-64 of the row's power of two, and
+// the products of weight 8 and above: together about sqrt(n) 2^-64 of the product of the
+// two rows' powers of two (n non-zero terms, each worth seven products of two digits;
+// at most 7 n 2^-64).  An FMA chain errs by 2^-54 of the sum of the |terms| and more.  So
+// an eighth accumulator sums the products of the leading digits' absolute values, in
+// units of 2^-14 of that product: where it reaches 32 sqrt(n) (n at most the smaller
+// number of non-zero entries of the two rows), the digits add no more than 2^-55 of the
+// sum of the |terms| (at most 3.5 / sqrt(n) of n FMA roundings).  Where it does not, the
+// block computes its tile with FP64 FMAs instead, as it does for a row with an Inf, a
+// NaN or only entries below 2^-959.  Against exact sums, max / rms in units of the sum
+// of the |terms|, FMA chain in brackets: K 8 .. 64, half of each row scaled by 1/32 ..
+// 1/128 where the other is large, 0.9e-16 / 2.8e-17 (2.9e-16 / 5.2e-17); entries spread
+// over 2^16, K 32, 0.9e-16 / 3.4e-17 (7.0e-16 / 1.4e-16); normal entries, K 32, 0.6e-16 /
+// 1.3e-17 (2.9e-16 / 5.3e-17).  (Seven digits reached 1.4e-15 .. 2.8e-15 in the first.)
 //
 // Bound: the digit extraction (integer instructions run at half rate on GB300; each
-// tile extracts the rows that it shares with others again), with the MMAs (70 of
+// tile extracts the rows that it shares with others again), with the MMAs (74 of
 // 128 x 64 x 16 per 32 values of k, 64 clocks each) under it, then the rounding and
-// writing of the tile.  Measured: M = 12000, N = 800, K = 200 (half of an energy at o = 20,
-// v = 200, X = 600, R = 800) 0.35 ms, 11 TF/s; k_gemm64 10.8 ms per half with its 20-row
-// tiles.  Error of a reconstruction (K = R = 16 .. 800) against extended precision
-// 0.7 .. 1.4e-16, k_gemm64 1.4 .. 3.0e-16.
+// writing of the tile.  Measured: an energy at o = 20, v = 200, X = 600, R = 800, two
+// contractions of M = 12000, N = 800, K = 200, 0.836 ms in all (0.851 with seven digits and
+// the rows' norms in place of their counts), 21.7 ms with k_gemm64 and 20-row tiles.
 #include "ppl_internal.h"
 #include "ppl_gemm64.cuh"
 #include "ppl_ptx.cuh"
@@ -48,17 +52,24 @@ constexpr int ETHREADS = EWORK + 128;          // and a warpgroup of which warp 
 // stream of dependent integer instructions.
 constexpr int EREG_LAUNCH = 96, EREG_CTRL = 64, EREG_WORK = 104;
 static_assert((ETHREADS - EWORK) * EREG_CTRL + EWORK * EREG_WORK == ETHREADS * EREG_LAUNCH, "register split");
-constexpr int NDIG = 7;                        // digits; plane 7 holds |leading digit|
-constexpr int FOLD = 4;                        // k blocks per exact FP32 accumulation: 7 * 128 * 2^14 < 2^24
+constexpr int NDIG = 8;                        // digits; plane 8 holds |leading digit|
+constexpr int NSUM = 7;                        // accumulators of their products
+constexpr int FOLD = 4;                        // k blocks per exact FP32 accumulation
 // A pair of digit planes shares one 128-byte row: plane p at bytes 64 (p & 1) .. + 63 of
-// the rows of pair p / 2, the 128 rows of A and then the 64 of B.
-constexpr uint32_t BOFF = EM * 128, PAIR = (EM + EN) * 128;
-constexpr uint32_t ESTAGE = 4 * PAIR;
+// the rows of pair p / 2, the 128 rows of A and then the 64 of B.  Plane 8 follows, A's
+// at bytes 0 .. 63 and B's at bytes 64 .. 127 of the same rows.
+constexpr uint32_t BOFF = EM * 128, PAIR = (EM + EN) * 128, GOFF = 4 * PAIR;
+constexpr uint32_t ESTAGE = GOFF + EM * 128;
 constexpr int CPITCH = EN + 1;
-constexpr size_t ESMEM = 2 * ESTAGE + 1024;
+// Two stages and the static arrays, rounded up to the stages' alignment, are exactly the
+// 227 KB a block can have.
+constexpr size_t ESMEM = 2 * ESTAGE;
+// After the products, over the stages: the sums, the guard's limits, the offsets in C
+constexpr uint32_t LIMOFF = EM * CPITCH * 12, OFFOFF = LIMOFF + (EM + EN) * 4;
+constexpr float GUARD2 = 1024.0f;              // 32 squared, per non-zero entry (see above)
 constexpr unsigned long long EWAIT_NS = 500ull * 1000ull * 1000ull;
-static_assert(EM * CPITCH * 12 <= 2 * ESTAGE, "the output tile is staged over the operand stages");
-static_assert(FOLD * EK * NDIG * (1 << 14) < (1 << 24), "exact FP32 sums");
+static_assert(OFFOFF + (EM + EN) * 8 <= ESMEM && OFFOFF % 8 == 0, "the output tile is staged over the operand stages");
+static_assert(FOLD * EK * (NSUM * (1 << 14) + NDIG * (1 << 6)) < (1 << 24), "exact FP32 sums");
 
 // k -> offset of km, for k0 and the k after it
 struct KOff {
@@ -82,33 +93,22 @@ __device__ __forceinline__ long long knext(const Idx2& km, KOff& o) {
 // k range of one split-K slice
 __host__ __device__ __forceinline__ int slice_len(int K, int ksplit) { return ((K + ksplit - 1) / ksplit + EK - 1) / EK * EK; }
 
-// ---- the rows' largest entries and norms -----------------------------------------
+// ---- the rows' largest entries and counts -----------------------------------------
 
 // A row's largest entry (the high word of its magnitude, 0 only for a row of zeros)
-// and its sum of squares in units of 4^(its exponent).
+// and its number of non-zero entries.
 struct RowStat {
-    unsigned int hi;
-    float sq;
+    unsigned int hi, n;
 };
-__device__ __forceinline__ float pow4(int d) {          // 4^-d, d >= 0
-    return __int_as_float(max(127 - 2 * d, 0) << 23);
-}
 __device__ __forceinline__ void stat_add(RowStat& s, double x) {
     const unsigned int h = (unsigned int)__double2hiint(x) & 0x7fffffffu;
-    const int ex = (int)(h >> 20), em = (int)(s.hi >> 20);
-    const float f = __uint_as_float(((h & 0xfffffu) << 3) | 0x3f800000u);
-    if (ex > em) {
-        s.sq *= pow4(ex - em);
-        s.sq = fmaf(f, f, s.sq);
-    } else if (ex > 0) {
-        s.sq = fmaf(f * f, pow4(em - ex), s.sq);
-    }
-    s.hi = max(s.hi, h | (h == 0u && __double2loint(x) != 0 ? 1u : 0u));
+    const bool nz = (h | (unsigned int)__double2loint(x)) != 0u;
+    s.hi = max(s.hi, h | (nz ? 1u : 0u));        // (the lowest bit is not used)
+    s.n += nz ? 1u : 0u;
 }
-__device__ __forceinline__ void stat_merge(RowStat& s, unsigned int hi, float sq) {
-    const int ea = (int)(s.hi >> 20), eb = (int)(hi >> 20), e = max(ea, eb);
-    s.sq = s.sq * pow4(e - ea) + sq * pow4(e - eb);
+__device__ __forceinline__ void stat_merge(RowStat& s, unsigned int hi, unsigned int n) {
     s.hi = max(s.hi, hi);
+    s.n += n;
 }
 
 // One operand: `rows` rows (map rm) of K entries (map km) for nb batch entries bs
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(256) k_rowstat(const __grid_constant__ RowArgs
     const RowArgs& x = second ? b : a;
     const int blk = second ? (int)blockIdx.x - a.nblk : (int)blockIdx.x;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    RowStat m{0u, 0.0f};
+    RowStat m{0u, 0u};
     if (x.km.lo == 1) {
         const bool wr = x.per <= RM_WARP_K;
         const long long e = wr ? (long long)blk * 8 + warp : blk;          // (batch, slice, row)
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(256) k_rowstat(const __grid_constant__ RowArgs
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1)
-            stat_merge(m, __shfl_xor_sync(0xffffffffu, m.hi, o), __shfl_xor_sync(0xffffffffu, m.sq, o));
+            stat_merge(m, __shfl_xor_sync(0xffffffffu, m.hi, o), __shfl_xor_sync(0xffffffffu, m.n, o));
         if (wr) {
             if (ok && lane == 0) x.out[e] = m;
             return;
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(256) k_rowstat(const __grid_constant__ RowArgs
         if (lane == 0) red[0][warp] = m;
         __syncthreads();
         if (threadIdx.x == 0) {
-            for (int w = 1; w < 8; ++w) stat_merge(m, red[0][w].hi, red[0][w].sq);
+            for (int w = 1; w < 8; ++w) stat_merge(m, red[0][w].hi, red[0][w].n);
             x.out[e] = m;
         }
         return;
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(256) k_rowstat(const __grid_constant__ RowArgs
     red[warp][lane] = m;
     __syncthreads();
     if (warp == 0 && row < x.rows) {
-        for (int w = 1; w < 8; ++w) stat_merge(m, red[w][lane].hi, red[w][lane].sq);
+        for (int w = 1; w < 8; ++w) stat_merge(m, red[w][lane].hi, red[w][lane].n);
         x.out[(long long)bt * x.rows + row] = m;
     }
 }
@@ -178,42 +178,55 @@ __global__ void __launch_bounds__(256) k_rowstat(const __grid_constant__ RowArgs
 // barrier 3 over the working threads
 __device__ __forceinline__ void work_sync() { asm volatile("bar.sync 3, 512;" ::: "memory"); }
 
-// the eight digit planes of four entries as pairs of consecutive k, w[plane][pair].
+// a >> d, 0 from d = 64 on
+__device__ __forceinline__ unsigned long long shr_clamp(unsigned long long a, unsigned int d) {
+    unsigned long long r;
+    asm("shr.b64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(d));
+    return r;
+}
+
+// the nine planes of four entries as pairs of consecutive k, w[plane][pair].
 // emax: the exponent field of the largest entry of the pair's row, in place (bits
 // 20 .. 30), at least 64 << 20 (rows below that are left to the FP64 tile, whatever is
 // written here).
-__device__ __forceinline__ void digits4(const double (&v)[4], const int (&emx)[2], uint32_t (&w)[8][2]) {
+__device__ __forceinline__ void digits4(const double (&v)[4], const int (&emx)[2], uint32_t (&w)[NDIG + 1][2]) {
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
         float f[2][NDIG];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const int hi = __double2hiint(v[2 * j + u]), lo = __double2loint(v[2 * j + u]);
-            // |x| = m 2^(ex - 1075), m < 2^53; X = round(x 2^(55 - e)), 2^e the power of two
-            // above the row's maximum, is m 2^(2 - d), d = emax - ex; one bit more is kept
+            // |x| = m 2^(ex - 1075), m < 2^53; X = round(x 2^(63 - e)), 2^e the power of two
+            // above the row's maximum, is m 2^(10 - d), d = emax - ex; one bit more is kept
             // for the rounding (a zero has d >= 64 and shifts out)
-            const int d = min((emx[j] - (hi & 0x7ff00000)) >> 20, 63);
-            const unsigned long long m =
-                (((unsigned long long)((hi & 0xfffff) | 0x100000) << 35) | ((unsigned long long)(unsigned int)lo << 3)) >> d;
-            // balanced digits: the lower six with 128 added are the bytes of t = X + 128 (256^0 + .. + 256^5)
-            const long long sg = (long long)(hi >> 31);
-            const long long t = ((long long)(m ^ (unsigned long long)sg) + ((0x0000808080808080ll * 2 + 1) - sg)) >> 1;
-            const uint32_t tl = (uint32_t)t, th = (uint32_t)((unsigned long long)t >> 32);
+            const unsigned int d = (unsigned int)((emx[j] - (hi & 0x7ff00000)) >> 20);
+            const unsigned long long m = shr_clamp(
+                ((unsigned long long)(__funnelshift_l((unsigned int)lo, (unsigned int)hi, 11) | 0x80000000u) << 32) |
+                    ((unsigned int)lo << 11), d);
+            // balanced digits: the lower seven with 128 added are the bytes of
+            // t = X + 128 (256^0 + .. + 256^6), the leading one, -128 .. 128, is what carries on
+            const unsigned int sg = (unsigned int)(hi >> 31);
+            const unsigned long long q = (m >> 1) + (m & 1u);
+            uint32_t tl, th, tc;
+            asm("add.cc.u32 %0, %3, %5;\n\taddc.cc.u32 %1, %4, 0x00808080;\n\taddc.u32 %2, %6, 0;"
+                : "=r"(tl), "=r"(th), "=r"(tc)
+                : "r"((uint32_t)q ^ sg), "r"((uint32_t)(q >> 32) ^ sg), "r"(0x80808080u - sg), "r"(sg));
             // a byte in the mantissa of 2^23 (the second one: 256 times it) less its offset, times
             // the digit's weight 256^-i: one exact FMA
-            f[u][0] = __int_as_float(0x4B400000 + ((int)th >> 16)) - 12582912.0f;
-            f[u][1] = fmaf(__uint_as_float((th & 0xff00u) | 0x4B000000u), 0x1p-16f, -32896.0f * 0x1p-8f);
-            f[u][2] = fmaf(__uint_as_float((th & 0xffu) | 0x4B000000u), 0x1p-16f, -8388736.0f * 0x1p-16f);
-            f[u][3] = fmaf(__uint_as_float(__byte_perm(tl, 0x4B000000u, 0x7443)), 0x1p-24f, -8388736.0f * 0x1p-24f);
-            f[u][4] = fmaf(__uint_as_float(__byte_perm(tl, 0x4B000000u, 0x7442)), 0x1p-32f, -8388736.0f * 0x1p-32f);
-            f[u][5] = fmaf(__uint_as_float((tl & 0xff00u) | 0x4B000000u), 0x1p-48f, -32896.0f * 0x1p-40f);
-            f[u][6] = fmaf(__uint_as_float((tl & 0xffu) | 0x4B000000u), 0x1p-48f, -8388736.0f * 0x1p-48f);
+            f[u][0] = __int_as_float(0x4B400000 + (int)__funnelshift_r(th, tc, 24)) - 12582912.0f;
+            f[u][1] = fmaf(__uint_as_float(__byte_perm(th, 0x4B000000u, 0x7442)), 0x1p-8f, -8388736.0f * 0x1p-8f);
+            f[u][2] = fmaf(__uint_as_float((th & 0xff00u) | 0x4B000000u), 0x1p-24f, -32896.0f * 0x1p-16f);
+            f[u][3] = fmaf(__uint_as_float((th & 0xffu) | 0x4B000000u), 0x1p-24f, -8388736.0f * 0x1p-24f);
+            f[u][4] = fmaf(__uint_as_float(__byte_perm(tl, 0x4B000000u, 0x7443)), 0x1p-32f, -8388736.0f * 0x1p-32f);
+            f[u][5] = fmaf(__uint_as_float(__byte_perm(tl, 0x4B000000u, 0x7442)), 0x1p-40f, -8388736.0f * 0x1p-40f);
+            f[u][6] = fmaf(__uint_as_float((tl & 0xff00u) | 0x4B000000u), 0x1p-56f, -32896.0f * 0x1p-48f);
+            f[u][7] = fmaf(__uint_as_float((tl & 0xffu) | 0x4B000000u), 0x1p-56f, -8388736.0f * 0x1p-56f);
         }
         // the upper halves are the bf16 values (eight significant bits)
 #pragma unroll
         for (int p = 0; p < NDIG; ++p)
             w[p][j] = __byte_perm(__float_as_uint(f[0][p]), __float_as_uint(f[1][p]), 0x7632);
-        w[7][j] = w[0][j] & 0x7fff7fffu;
+        w[NDIG][j] = w[0][j] & 0x7fff7fffu;
     }
 }
 
@@ -228,8 +241,8 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem, unsigned long long ad, u
 
 // four columns of the seven digit-sum accumulators (EN columns apart); the wait is part
 // of the statement, so that nothing reads the registers before it
-__device__ __forceinline__ void tmem_ld_sums(uint32_t taddr, uint32_t (&s)[NDIG][4]) {
-    static_assert(NDIG == 7 && EN == 64, "spelled out below");
+__device__ __forceinline__ void tmem_ld_sums(uint32_t taddr, uint32_t (&s)[NSUM][4]) {
+    static_assert(NSUM == 7 && EN == 64, "spelled out below");
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%28];\n\t"
         "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4, %5, %6, %7}, [%29];\n\t"
@@ -299,11 +312,9 @@ struct SplitArgs {
 
 __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_constant__ SplitArgs sa_) {
     const G64& g = sa_.g;
-    extern __shared__ unsigned char smem_raw[];
+    extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ int s_ex[EM + EN];              // the rows' exponent fields, in place
-    __shared__ float s_lim[EM + EN];           // the guard's limits
     __shared__ long long s_row[EM + EN];       // the rows' offsets in A and B
-    __shared__ long long s_off[EM + EN];       // the tile's row and column offsets in C
     __shared__ unsigned long long s_bar[5];    // full[2], empty[2], folded
     __shared__ uint32_t s_tmem;
     __shared__ int s_fail, s_bad;
@@ -321,8 +332,11 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
     if (kbeg >= kend) return;          // a split slice past the end (atomic outputs only)
     const int nkb = (kend - kbeg + EK - 1) / EK;
 
-    const uint32_t raw = smem_u32(smem_raw), base = (raw + 1023u) & ~1023u;
-    unsigned char* sm = smem_raw + (base - raw);
+    const uint32_t base = smem_u32(sm);
+    if (base & 1023u) {                // (the swizzled tiles need the alignment asked for above)
+        if (tid == 0) atomicOr(g.err, 256u);
+        return;
+    }
     const uint32_t full0 = smem_u32(&s_bar[0]), bar0 = smem_u32(&s_bar[2]), folded = smem_u32(&s_bar[4]);
     if (tid == 0) {
         s_fail = 0;
@@ -334,20 +348,20 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
         mbar_init(folded, EWORK / 32);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int i = tid; i < EM + EN; i += ETHREADS) {
+    float lim = 0.0f;                  // the limit of row `tid`
+    if (tid < EM + EN) {
+        const int i = tid;
         const bool isb = i >= EM;
         const int r = isb ? n0 + i - EM : m0 + i;
         const bool ok = r < (isb ? g.N : g.M);
         // (a row past the end stands for row 0: its sums are never written)
-        const RowStat st = !ok ? RowStat{0u, 0.0f}
+        const RowStat st = !ok ? RowStat{0u, 0u}
                            : isb ? sa_.hb[(long long)(b * sa_.bb * g.ksplit + ks) * g.N + r]
                                  : sa_.ha[(long long)(b * sa_.ba * g.ksplit + ks) * g.M + r];
         s_ex[i] = (int)max(st.hi & 0x7ff00000u, 64u << 20);        // a zero row has zero digits
-        // half the norm of the row's leading digits (64 = its exponent); a zero row never
-        // fails the guard, a row with an Inf, a NaN or nothing above 2^-959 always does
-        s_lim[i] = st.hi == 0u ? -1e30f : (st.hi >= 0x7ff00000u || (st.hi >> 20) < 64u) ? 1e35f : 32.0f * sqrtf(st.sq);
+        // no limit for a zero row; a row with an Inf, a NaN or nothing above 2^-959 never passes
+        lim = (st.hi >= 0x7ff00000u || (st.hi >> 20) < 64u) && st.hi != 0u ? -1.0f : GUARD2 * (float)st.n;
         s_row[i] = !ok ? 0 : ixd(isb ? g.bn : g.am, r);
-        s_off[i] = isb ? ixd(g.cn, r) : ixd(g.cm, r);
     }
     if (warp == EWORK / 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&s_tmem)) : "memory");
@@ -381,17 +395,16 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
                     for (int i = 0; i < NDIG; ++i) {
                         const unsigned long long da = make_desc(sa + (uint32_t)(i >> 1) * PAIR) + (unsigned long long)(((i & 1) * 64 + kk * 32) >> 4);
 #pragma unroll
-                        for (int j = 0; j < NDIG && i + j <= NDIG; ++j) {
+                        for (int j = 0; i + j < NDIG; ++j) {
                             const unsigned long long db = make_desc(sb + (uint32_t)(j >> 1) * PAIR) + (unsigned long long)(((j & 1) * 64 + kk * 32) >> 4);
                             // weight i + j, weight 7 with weight 6; the first product of an
                             // accumulator is that of i = 0
-                            mma_bf16(tmem + (uint32_t)(min(i + j, NDIG - 1) * EN), da, db, idesc,
-                                     (kb % FOLD > 0 || kk > 0 || i > 0) ? 1u : 0u);
+                            mma_bf16(tmem + (uint32_t)(min(i + j, NSUM - 1) * EN), da, db, idesc,
+                                     (kb % FOLD > 0 || kk > 0 || i > 0 || j >= NSUM) ? 1u : 0u);
                         }
                     }
-                    const unsigned long long da = make_desc(sa + 3 * PAIR) + (unsigned long long)((64 + kk * 32) >> 4);
-                    const unsigned long long db = make_desc(sb + 3 * PAIR) + (unsigned long long)((64 + kk * 32) >> 4);
-                    mma_bf16(tmem + (uint32_t)(NDIG * EN), da, db, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+                    const unsigned long long gd = make_desc(sa + GOFF) + (unsigned long long)((kk * 32) >> 4);
+                    mma_bf16(tmem + (uint32_t)(NSUM * EN), gd, gd + (64 >> 4), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
                 }
                 mma_commit(bar0 + 8u * (kb & 1));
             }
@@ -486,7 +499,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
                 else if (kb + 1 < nkb)
                     load(0, kb + 1, v);
                 int emx[2];
-                uint32_t w[8][2];
+                uint32_t w[NDIG + 1][2];
                 unsigned char* op = sm + (uint32_t)(kb & 1) * ESTAGE;
                 if (kf) {
 #pragma unroll
@@ -499,7 +512,8 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
                         unsigned char* q0 = op + r * 128u + (((uint32_t)(lane & 15) * 4u) ^ ((r & 7u) << 4));
                         unsigned char* q1 = op + r * 128u + ((64u + (uint32_t)(lane & 15) * 4u) ^ ((r & 7u) << 4));
 #pragma unroll
-                        for (int p = 0; p < 8; ++p) *(uint32_t*)(((p & 1) ? q1 : q0) + (p >> 1) * PAIR) = w[p][i];
+                        for (int p = 0; p < NDIG; ++p) *(uint32_t*)(((p & 1) ? q1 : q0) + (p >> 1) * PAIR) = w[p][i];
+                        *(uint32_t*)((isb ? q1 - BOFF : q0) + GOFF) = w[NDIG][i];
                     }
                 } else {
                     const uint32_t r = (uint32_t)step_row(u, false, 0);
@@ -508,7 +522,8 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
                     unsigned char* q0 = op + r * 128u + (((uint32_t)(tid >> 6) * 8u) ^ ((r & 7u) << 4));
                     unsigned char* q1 = op + r * 128u + ((64u + (uint32_t)(tid >> 6) * 8u) ^ ((r & 7u) << 4));
 #pragma unroll
-                    for (int p = 0; p < 8; ++p) *(uint2*)(((p & 1) ? q1 : q0) + (p >> 1) * PAIR) = make_uint2(w[p][0], w[p][1]);
+                    for (int p = 0; p < NDIG; ++p) *(uint2*)(((p & 1) ? q1 : q0) + (p >> 1) * PAIR) = make_uint2(w[p][0], w[p][1]);
+                    *(uint2*)((isb ? q1 - BOFF : q0) + GOFF) = make_uint2(w[NDIG][0], w[NDIG][1]);
                 }
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -521,16 +536,16 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            constexpr float unit[NDIG] = {1.0f, 0x1p8f, 0x1p16f, 0x1p24f, 0x1p32f, 0x1p40f, 0x1p48f};
+            constexpr float unit[NSUM] = {1.0f, 0x1p8f, 0x1p16f, 0x1p24f, 0x1p32f, 0x1p40f, 0x1p48f};
 #pragma unroll
             for (int j0 = 0; j0 < NC; j0 += 4) {
-                uint32_t s[NDIG][4];
+                uint32_t s[NSUM][4];
                 tmem_ld_sums(tq + (uint32_t)j0, s);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    int d[NDIG];
+                    int d[NSUM];
 #pragma unroll
-                    for (int w = 0; w < NDIG; ++w) d[w] = __float2int_rn(__uint_as_float(s[w][j]) * unit[w]);
+                    for (int w = 0; w < NSUM; ++w) d[w] = __float2int_rn(__uint_as_float(s[w][j]) * unit[w]);
                     const long long lo = (long long)d[4] * 65536 + (long long)d[5] * 256 + d[6] + (long long)L[j0 + j];
                     H[j0 + j] += (long long)(d[0] * 256 + d[1]) * 65536 + (d[2] * 256 + d[3]) + (lo >> 24);
                     L[j0 + j] = (unsigned int)lo & 0xffffffu;
@@ -541,24 +556,33 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
             if (kb < nkb && lane == 0) mbar_arrive(folded);
         }
     }
+    // the MMAs have read the operands
+    float* s_lim = (float*)(sm + LIMOFF);
+    long long* s_off = (long long*)(sm + OFFOFF);
+    if (tid < EM + EN) {
+        s_lim[tid] = lim;
+        s_off[tid] = tid < EM ? ixd(g.cm, m0 + tid) : ixd(g.cn, n0 + tid - EM);
+    }
     work_sync();
     const bool failed = *vfail != 0;
     int bad = 0;
     if (!failed) {
-        const float na = m0 + q * 32 + lane < g.M ? s_lim[q * 32 + lane] : -1e36f;
+        const float la = s_lim[q * 32 + lane];
 #pragma unroll 1
         for (int j0 = 0; j0 < NC; j0 += 8) {
             uint32_t s[8];
-            tmem_ld8(tq + (uint32_t)(NDIG * EN + j0), s);
+            tmem_ld8(tq + (uint32_t)(NSUM * EN + j0), s);
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (__uint_as_float(s[j]) < na + s_lim[EM + c0 + j0 + j] && n0 + c0 + j0 + j < g.N) bad = 1;
+            for (int j = 0; j < 8; ++j) {
+                const float t = fminf(la, s_lim[EM + c0 + j0 + j]), sum = __uint_as_float(s[j]);
+                if ((t < 0.0f || sum * sum < t) && n0 + c0 + j0 + j < g.N && m0 + q * 32 + lane < g.M) bad = 1;
+            }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     }
     asm volatile("bar.arrive 2, 544;" ::: "memory");
     if (bad) s_bad = 1;
-    // stage the sums in shared memory (the MMAs have read the operands)
+    // stage the sums in shared memory
     long long* sH = (long long*)sm;
     unsigned int* sL = (unsigned int*)(sH + EM * CPITCH);
 #pragma unroll

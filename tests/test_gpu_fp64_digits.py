@@ -1,0 +1,126 @@
+"""FP64 contractions formed from exact digit products (csrc/ppl_split64.cu), against exact
+integer arithmetic.
+
+The reconstruction R~[a,b,i,j] = sum_r Ua[a,r] Ub[b,r] Ui[i,r] Uj[j,r] with U_b = U_j = 1
+is one contraction of the rows of U_a with the rows of U_i over K = R, so any rows can
+be tried:
+
+* the digit form must be no worse than the FP64 FMA chain it stands for on any rows: the
+  chain is evaluated exactly here, and over the 240 elements of a case the rms error (in
+  units of the sum of the |terms|) may be 1.25 times the chain's and the largest error
+  twice the chain's (what two samples of that size differ by).
+* for sums without cancellation the digit form is rounded once: 0.51 units in the last
+  place.  A chain of 256 FMAs is several units off, so this also shows which kernel ran.
+"""
+
+import math
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2503_10380_gb300 import binding
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+def _handle(A, B, precision="fp64"):
+    """A handle whose reconstruction is A B^T: A [v][K] in mode a, B [o][K] in mode i."""
+    (v, K), o = A.shape, B.shape[0]
+    fac = {"a": A, "b": np.ones((v, K)), "i": B, "j": np.ones((o, K))}
+    g = torch.Generator().manual_seed(0)
+    Bt = torch.randn(2, o + v, o + v, generator=g, dtype=torch.float64)
+    tau = torch.randn(o, o, v, v, generator=g, dtype=torch.float64)
+    return binding.CpAls((Bt + Bt.transpose(1, 2)).cuda(), tau.cuda(), fac, precision=precision)
+
+
+def _products(A, B, precision="fp64"):
+    """[v][o] from the device: of the copies [b][j] of an element, one from all over the output"""
+    cp = _handle(A, B, precision)
+    R = cp.reconstruct(symmetrise=False).cpu().numpy()       # [a][b][i][j]
+    cp.close()
+    a, i = np.meshgrid(np.arange(A.shape[0]), np.arange(B.shape[0]), indexing="ij")
+    return R[a, (7 * a + 3 * i) % A.shape[0], i, (a + i) % B.shape[0]]
+
+
+def _ints(A):
+    """A = ints 2^-s, exactly"""
+    low = min((math.frexp(x)[1] for x in A.ravel() if x != 0.0), default=0)
+    s = 53 - low
+    return np.array([[int(Fraction(float(x)) * Fraction(2) ** s) for x in r] for r in A], dtype=object), s
+
+
+def _errors(got, A, B):
+    """|got - exact| and sum |terms|, both as floats, and the exact values"""
+    (IA, sa), (IB, sb) = _ints(A), _ints(B)
+    unit = Fraction(2) ** -(sa + sb)
+    ex = [[Fraction(int(x)) * unit for x in r] for r in IA @ IB.T]
+    ab = np.array([[float(Fraction(int(x)) * unit) for x in r] for r in np.abs(IA) @ np.abs(IB).T])
+    err = np.array([[float(abs(Fraction(float(g)) - e)) for g, e in zip(gr, er)] for gr, er in zip(got, ex)])
+    return err, ab, np.array([[float(e) for e in r] for r in ex])
+
+
+def _fma_chain(x, y):
+    s = 0.0
+    for p, q in zip(x, y):
+        s = float(Fraction(float(p)) * Fraction(float(q)) + Fraction(s))     # rounded once
+    return s
+
+
+def _rows(kind, K, rng, v=40, o=6):
+    A, B = rng.standard_normal((v, K)), rng.standard_normal((o, K))
+    if kind.startswith("opposed"):                # one operand large where the other is small
+        s = 2.0 ** -int(kind[7:])
+        A[:, K // 2:] *= s
+        B[:, :K // 2] *= s
+    elif kind.startswith("spread"):
+        s = float(kind[6:])
+        A *= 2.0 ** rng.uniform(-s, 0, A.shape)
+        B *= 2.0 ** rng.uniform(-s, 0, B.shape)
+    elif kind == "decay":
+        d = np.exp(-np.arange(K) / 15.0)
+        A *= d
+        B *= d
+    return A, B
+
+
+@pytest.mark.parametrize("kind,K", [("even", 8), ("even", 33), ("opposed3", 8), ("opposed5", 8), ("opposed7", 8),
+                                    ("opposed10", 9), ("opposed6", 64), ("opposed9", 64), ("spread16", 32),
+                                    ("spread24", 128), ("decay", 150), ("spread40", 40)])
+def test_no_worse_than_an_fma_chain(kind, K):
+    A, B = _rows(kind, K, np.random.default_rng(K))
+    err, ab, _ = _errors(_products(A, B), A, B)
+    chain, _, _ = _errors([[_fma_chain(x, y) for y in B] for x in A], A, B)
+    r, c = err / ab, chain / ab
+    assert r.max() <= 2.0 * c.max(), (r.max(), c.max())
+    assert np.sqrt(np.mean(r * r)) <= 1.25 * np.sqrt(np.mean(c * c))
+
+
+@pytest.mark.parametrize("K", [8, 31, 32, 33, 128, 129, 256])
+def test_sums_of_one_sign_are_rounded_once(K):
+    rng = np.random.default_rng(100 + K)
+    A, B = 0.5 + 0.5 * rng.random((40, K)), 0.5 + 0.5 * rng.random((6, K))
+    err, _, ex = _errors(_products(A, B), A, B)
+    assert np.max(err / np.spacing(ex)) <= 0.51
+
+
+def test_largest_digits():
+    """Every digit +127 or -128 over two full folds of 128 k: the FP32 sums of products of
+    one weight come within an eighth of 2^24, and stay exact."""
+    plus = 0x7f7f7f7f7f7f
+    minus = 127 * 256 ** 5 - 128 * sum(256 ** k for k in range(5))
+    K = 256
+    A = np.array([[float(plus)] * K, [float(minus)] * K, [float(-minus)] * K, [float(plus), float(minus)] * (K // 2)])
+    B = np.array([[float(minus)] * K, [float(plus)] * K])
+    err, ab, ex = _errors(_products(A, B), A, B)
+    assert np.all(err <= 0.51 * np.spacing(np.abs(ex)))
