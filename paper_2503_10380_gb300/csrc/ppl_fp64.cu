@@ -20,7 +20,7 @@ __global__ void __launch_bounds__(256) k_gemm64(const __grid_constant__ G64 g) {
     const int kbeg = ks * per, kend = min(g.K, kbeg + per);
     if (kbeg >= kend && g.atomic) return;
     __shared__ double sm[GBK * (GBM + GBN)];
-    gemm64_tile(g, b, m0, n0, kbeg, kend, sm);
+    gemm64_tile(g, b, m0, n0, kbeg, kend, sm, threadIdx.x, 1);
 }
 
 __global__ void k_kr(const double* Ui, const double* Uj, int o, int R, double* KR, int ld) {

@@ -12,17 +12,18 @@ __device__ __forceinline__ long long ixd(const Idx2& x, int i) {
     return (long long)(i / x.div) * x.hi + (long long)(i % x.div) * x.lo;
 }
 
-// barrier 1 over the 256 threads of the tile (a caller's block may have more)
-__device__ __forceinline__ void block_sync256() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+// barrier `bar` over the 256 threads of the tile (a caller's block may have more)
+__device__ __forceinline__ void block_sync256(int bar) { asm volatile("bar.sync %0, 256;" ::"r"(bar) : "memory"); }
 
-// Rows m0 .., columns n0 .. of batch entry b over kbeg .. kend - 1: 256 threads, 4 x 4
+// Rows m0 .., columns n0 .. of batch entry b over kbeg .. kend - 1: 256 threads (tid), 4 x 4
 // outputs per thread at (ty + 16 i, tx + 16 j), sm: GBK (GBM + GBN) doubles of shared
-// memory.  Operands are read through Idx2 maps, so every layout of the method is
+// memory, bar: a barrier of their own.  Operands are read through Idx2 maps, so every layout of the method is
 // served without copies; the FP64 pipe (not the loads) bounds it on GB300.
-__device__ __forceinline__ void gemm64_tile(const G64& g, int b, int m0, int n0, int kbeg, int kend, double* sm) {
+__device__ __forceinline__ void gemm64_tile(const G64& g, int b, int m0, int n0, int kbeg, int kend, double* sm, int tid,
+                                            int bar) {
     double(*As)[GBM] = (double(*)[GBM])sm;
     double(*Bs)[GBN] = (double(*)[GBN])(sm + GBK * GBM);
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+    const int tx = tid % 16, ty = tid / 16;
     const double* A = g.A + (long long)b * g.ab;
     const double* B = g.B + (long long)b * g.bb;
     const bool a_kfast = (g.ak.lo == 1 && g.ak.div >= (1 << 30));
@@ -56,7 +57,7 @@ __device__ __forceinline__ void gemm64_tile(const G64& g, int b, int m0, int n0,
             As[a_kl[q]][a_ml[q]] = (a_row[q] >= 0 && ka < kend) ? A[a_row[q] + ixd(g.ak, ka)] : 0.0;
             Bs[b_kl[q]][b_nl[q]] = (b_row[q] >= 0 && kb < kend) ? B[b_row[q] + ixd(g.bk, kb)] : 0.0;
         }
-        block_sync256();
+        block_sync256(bar);
 #pragma unroll
         for (int kk = 0; kk < GBK; ++kk) {
             double av[4], bv[4];
@@ -69,7 +70,7 @@ __device__ __forceinline__ void gemm64_tile(const G64& g, int b, int m0, int n0,
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
         }
-        block_sync256();
+        block_sync256(bar);
     }
 
     double* C = g.C + (long long)b * g.cb;

@@ -22,9 +22,10 @@
 // an eighth accumulator sums the products of the leading digits' absolute values, in
 // units of 2^-14 of that product: where it reaches 32 sqrt(n) (n at most the smaller
 // number of non-zero entries of the two rows), the digits add no more than 2^-55 of the
-// sum of the |terms| (at most 3.5 / sqrt(n) of n FMA roundings).  Where it does not, the
-// block computes its tile with FP64 FMAs instead, as it does for a row with an Inf, a
-// NaN or only entries below 2^-959.  Against exact sums, max / rms in units of the sum
+// sum of the |terms| (at most 3.5 / sqrt(n) of n FMA roundings).  An element for which it
+// does not is formed by FP64 FMAs, as are those of a row with an Inf, a NaN or only
+// entries below 2^-959; one whose terms are all zero (the sum then is exactly zero) is
+// not.  Against exact sums, max / rms in units of the sum
 // of the |terms|, FMA chain in brackets: K 8 .. 64, half of each row scaled by 1/32 ..
 // 1/128 where the other is large, 0.9e-16 / 2.8e-17 (2.9e-16 / 5.2e-17); entries spread
 // over 2^16, K 32, 0.9e-16 / 3.4e-17 (7.0e-16 / 1.4e-16); normal entries, K 32, 0.6e-16 /
@@ -64,11 +65,22 @@ constexpr int CPITCH = EN + 1;
 // Two stages and the static arrays, rounded up to the stages' alignment, are exactly the
 // 227 KB a block can have.
 constexpr size_t ESMEM = 2 * ESTAGE;
-// After the products, over the stages: the sums, the guard's limits, the offsets in C
-constexpr uint32_t LIMOFF = EM * CPITCH * 12, OFFOFF = LIMOFF + (EM + EN) * 4;
+// After the products, over the stages: the sums, the guard's limits, the offsets in C, the
+// elements below their limit, and which entries are not zero, KBITS of every row at a time
+constexpr int KBITS = 1024;
+constexpr uint32_t LIMOFF = EM * CPITCH * 12, OFFOFF = LIMOFF + (EM + EN) * 4, BADOFF = OFFOFF + (EM + EN) * 8;
+// Up to this many of a tile's 8192 elements a warp forms each by FP64 FMAs (some 240 clocks
+// per element at K = 250), beyond it the block computes the whole tile (2 FMAs per clock).
+// Reconstruction at o 16, v 150, R 500, with the whole tile for any such element before:
+// rows with a tenth of their entries 4.74 -> 2.37 ms, of two symmetry blocks 2.38 -> 0.73,
+// all four factors with a tenth 6.44 -> 1.06, entries spread over 2^40 6.44 -> 6.08, full
+// rows 0.63 (k_gemm64: 5.72, whatever the entries).
+constexpr int MAXBAD = 2048;
+constexpr uint32_t BITOFF = BADOFF + MAXBAD * 2, BITPITCH = KBITS / 32 + 1;
+constexpr unsigned int LBAD = 0xffffffffu;     // in place of a low sum word: element below its limit
 constexpr float GUARD2 = 1024.0f;              // 32 squared, per non-zero entry (see above)
 constexpr unsigned long long EWAIT_NS = 500ull * 1000ull * 1000ull;
-static_assert(OFFOFF + (EM + EN) * 8 <= ESMEM && OFFOFF % 8 == 0, "the output tile is staged over the operand stages");
+static_assert(BITOFF + (EM + EN) * BITPITCH * 4 <= ESMEM && BITOFF % 4 == 0 && EM * EN <= 65536 && OFFOFF % 8 == 0, "the output tile is staged over the operand stages");
 static_assert(FOLD * EK * (NSUM * (1 << 14) + NDIG * (1 << 6)) < (1 << 24), "exact FP32 sums");
 
 // k -> offset of km, for k0 and the k after it
@@ -317,7 +329,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
     __shared__ long long s_row[EM + EN];       // the rows' offsets in A and B
     __shared__ unsigned long long s_bar[5];    // full[2], empty[2], folded
     __shared__ uint32_t s_tmem;
-    __shared__ int s_fail, s_bad;
+    __shared__ int s_fail, s_bad, s_zeros, s_empty;
 
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     const int ntm = (g.M + EM - 1) / EM, ntn = (g.N + EN - 1) / EN;
@@ -341,6 +353,8 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
     if (tid == 0) {
         s_fail = 0;
         s_bad = 0;
+        s_zeros = 0;
+        s_empty = 0;
         mbar_init(full0, EWORK / 32);
         mbar_init(full0 + 8, EWORK / 32);
         mbar_init(bar0, 1);
@@ -348,6 +362,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
         mbar_init(folded, EWORK / 32);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    __syncthreads();
     float lim = 0.0f;                  // the limit of row `tid`
     if (tid < EM + EN) {
         const int i = tid;
@@ -361,6 +376,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
         s_ex[i] = (int)max(st.hi & 0x7ff00000u, 64u << 20);        // a zero row has zero digits
         // no limit for a zero row; a row with an Inf, a NaN or nothing above 2^-959 never passes
         lim = (st.hi >= 0x7ff00000u || (st.hi >> 20) < 64u) && st.hi != 0u ? -1.0f : GUARD2 * (float)st.n;
+        if (st.n > 0u && st.n < (unsigned int)(kend - kbeg)) s_zeros = 1;
         s_row[i] = !ok ? 0 : ixd(isb ? g.bn : g.am, r);
     }
     if (warp == EWORK / 32) {
@@ -565,7 +581,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
     }
     work_sync();
     const bool failed = *vfail != 0;
-    int bad = 0;
+    unsigned int bad = 0u, empty = 0u;      // of this thread's columns: below the limit, a sum of zero
     if (!failed) {
         const float la = s_lim[q * 32 + lane];
 #pragma unroll 1
@@ -575,31 +591,68 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const float t = fminf(la, s_lim[EM + c0 + j0 + j]), sum = __uint_as_float(s[j]);
-                if ((t < 0.0f || sum * sum < t) && n0 + c0 + j0 + j < g.N && m0 + q * 32 + lane < g.M) bad = 1;
+                if ((t < 0.0f || sum * sum < t) && n0 + c0 + j0 + j < g.N) bad |= 1u << (j0 + j);
+                if (t > 0.0f && sum == 0.0f) empty |= 1u << (j0 + j);
             }
         }
+        if (m0 + q * 32 + lane >= g.M) bad = 0u;
+        empty &= bad;
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     }
     asm volatile("bar.arrive 2, 544;" ::: "memory");
-    if (bad) s_bad = 1;
+    if (s_zeros) {
+        // Sums whose terms are all exactly zero (rows of disjoint support) are zero as they
+        // stand: where rows have zeros, the guard's zero sums are looked through entry by entry.
+        if (empty) s_empty = 1;
+        work_sync();
+        uint32_t* s_bits = (uint32_t*)(sm + BITOFF);
+        for (int k0 = kbeg; k0 < kend && s_empty; k0 += KBITS) {
+            for (int i = warp; i < EM + EN; i += EWORK / 32) {
+                const double* p = i < EM ? A + s_row[i] : B + s_row[i];
+                const Idx2& km = i < EM ? g.ak : g.bk;
+                for (int k = k0; k < min(kend, k0 + KBITS); k += 32) {
+                    const bool nz = k + lane < kend && __double_as_longlong(__ldg(p + ixd(km, k + lane))) << 1 != 0;
+                    const unsigned int w = __ballot_sync(0xffffffffu, nz);
+                    if (lane == 0) s_bits[i * BITPITCH + (k - k0) / 32] = w;
+                }
+            }
+            work_sync();
+            for (unsigned int x = empty; x != 0u; x &= x - 1u) {
+                const int j = __ffs(x) - 1;
+                unsigned int any = 0u;
+                for (int w = 0; w < (min(kend - k0, KBITS) + 31) / 32; ++w)
+                    any |= s_bits[(q * 32 + lane) * BITPITCH + w] & s_bits[(EM + c0 + j) * BITPITCH + w];
+                if (any) empty &= ~(1u << j);
+            }
+            work_sync();
+        }
+        bad &= ~empty;
+    }
+    unsigned short* s_list = (unsigned short*)(sm + BADOFF);
+    if (bad) {
+        int at = atomicAdd(&s_bad, __popc(bad));
+        for (unsigned int x = bad; x != 0u && at < MAXBAD; x &= x - 1u, ++at)
+            s_list[at] = (unsigned short)((q * 32 + lane) * EN + c0 + __ffs(x) - 1);
+    }
     // stage the sums in shared memory
     long long* sH = (long long*)sm;
     unsigned int* sL = (unsigned int*)(sH + EM * CPITCH);
 #pragma unroll
     for (int j = 0; j < NC; ++j) {
         sH[(q * 32 + lane) * CPITCH + c0 + j] = H[j];
-        sL[(q * 32 + lane) * CPITCH + c0 + j] = L[j];
+        sL[(q * 32 + lane) * CPITCH + c0 + j] = (bad >> j) & 1u ? LBAD : L[j];
     }
     work_sync();
     if (failed) {
         if (tid == 0) atomicOr(g.err, 128u);
         return;
     }
-    if (s_bad) {
-        // FP64 FMAs for this tile, 256 threads
-        if (tid >= 256) return;
-        for (int h = 0; h < EM; h += 64)
-            if (m0 + h < g.M) gemm64_tile(g, b, m0 + h, n0, kbeg, kend, (double*)sm);
+    const int nbad = s_bad;
+    if (nbad > MAXBAD) {
+        // FP64 FMAs for this tile, 256 threads per 64 rows
+        const int h = tid / 256;
+        if (m0 + h * 64 < g.M)
+            gemm64_tile(g, b, m0 + h * 64, n0, kbeg, kend, (double*)sm + h * GBK * (GBM + GBN), tid % 256, h == 0 ? 1 : 4);
         return;
     }
     // round and write along the output's contiguous index
@@ -616,8 +669,9 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
             const int e = e0 + y * EWORK;
             const int ml = nfast ? e / EN : e % EM, nl = nfast ? e % EN : e / EM;
             const int ex = (s_ex[ml] >> 20) + (s_ex[EM + nl] >> 20) - (2 * 1022 + 62);
-            x[y] = fixed_to_double(sH[ml * CPITCH + nl], sL[ml * CPITCH + nl], ex);
-            p[y] = m0 + ml < g.M && n0 + nl < g.N ? C + s_off[ml] + s_off[EM + nl] : nullptr;
+            const unsigned int l = sL[ml * CPITCH + nl];
+            x[y] = fixed_to_double(sH[ml * CPITCH + nl], l, ex);
+            p[y] = m0 + ml < g.M && n0 + nl < g.N && l != LBAD ? C + s_off[ml] + s_off[EM + nl] : nullptr;
         }
         if (plain) {
 #pragma unroll
@@ -628,6 +682,17 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
             for (int y = 0; y < NE; ++y)
                 if (p[y]) write_scaled(g, p[y], x[y]);
         }
+    }
+    // elements below their limit: a warp each, lanes along k
+    for (int i = warp; i < nbad; i += EWORK / 32) {
+        const int ml = s_list[i] / EN, nl = s_list[i] % EN;
+        const double *a = A + s_row[ml], *bp = B + s_row[EM + nl];
+        double x = 0.0;
+#pragma unroll 4
+        for (int k = kbeg + lane; k < kend; k += 32) x = fma(__ldg(a + ixd(g.ak, k)), __ldg(bp + ixd(g.bk, k)), x);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == 0) write_scaled(g, C + s_off[ml] + s_off[EM + nl], x);
     }
 }
 

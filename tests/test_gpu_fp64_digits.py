@@ -96,7 +96,8 @@ def _rows(kind, K, rng, v=40, o=6):
 
 @pytest.mark.parametrize("kind,K", [("even", 8), ("even", 33), ("opposed3", 8), ("opposed5", 8), ("opposed7", 8),
                                     ("opposed10", 9), ("opposed6", 64), ("opposed9", 64), ("spread16", 32),
-                                    ("spread24", 128), ("decay", 150), ("spread40", 40)])
+                                    ("spread24", 128), ("decay", 150), ("spread40", 40),
+                                    ("spread24", 300)])
 def test_no_worse_than_an_fma_chain(kind, K):
     A, B = _rows(kind, K, np.random.default_rng(K))
     err, ab, _ = _errors(_products(A, B), A, B)
@@ -124,3 +125,55 @@ def test_largest_digits():
     B = np.array([[float(minus)] * K, [float(plus)] * K])
     err, ab, ex = _errors(_products(A, B), A, B)
     assert np.all(err <= 0.51 * np.spacing(np.abs(ex)))
+
+
+@pytest.mark.parametrize("kind", ["random", "halves", "one", "wide"])
+@pytest.mark.parametrize("K", [33, 200, 300])
+def test_rows_with_zeros(kind, K):
+    """Rows with few non-zero entries: a sum without a non-zero term is exactly zero, the
+    others are as accurate as an FMA chain.  "wide": among the entries are some 2^-70 times
+    the others, which the digits cannot hold."""
+    rng = np.random.default_rng(7 * K + len(kind))
+    A, B = rng.standard_normal((40, K)), rng.standard_normal((6, K))
+    if kind == "halves":                 # supports of symmetry blocks
+        A[::2, K // 2:] = 0.0
+        A[1::2, :K // 2] = -0.0
+        B[::2, K // 2:] = 0.0
+        B[1::2, :K // 2] = 0.0
+    elif kind == "one":
+        A *= np.arange(K)[None] % 20 == np.arange(40)[:, None] % 20
+        B *= np.arange(K)[None] % 20 == np.arange(6)[:, None]
+    else:
+        A *= rng.random(A.shape) < 0.1
+        B *= rng.random(B.shape) < 0.1
+        if kind == "wide":
+            A *= np.where(rng.random(A.shape) < 0.5, 2.0 ** -70, 1.0)
+    got = _products(A, B)
+    err, ab, _ = _errors(got, A, B)
+    assert np.all(got[ab == 0.0] == 0.0) and np.any(ab == 0.0) and np.any(ab > 0.0)
+    chain, _, _ = _errors([[_fma_chain(x, y) for y in B] for x in A], A, B)
+    r, c = err[ab > 0] / ab[ab > 0], chain[ab > 0] / ab[ab > 0]
+    assert r.max() <= max(2.0 * c.max(), 2.0 ** -52)      # (few terms: an element is off by one rounding or two)
+
+
+def test_cost_of_rows_with_zeros():
+    """Nine in ten entries zero: a tenth of the elements is left to FP64 FMAs, the sums
+    without a term are not.  Within six times the time of full rows (all tiles by FMAs
+    take ten times and more)."""
+    v, o, K = 150, 12, 400
+    rng = np.random.default_rng(2)
+    ms = []
+    for density in (1.1, 0.1):
+        A, B = rng.standard_normal((v, K)), rng.standard_normal((o, K))
+        cp = _handle(A * (rng.random(A.shape) < density), B * (rng.random(B.shape) < density))
+        best = math.inf
+        for _ in range(8):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            cp.reconstruct(symmetrise=False)
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1))
+        ms.append(best)
+        cp.close()
+    assert ms[1] <= 6.0 * ms[0], ms
