@@ -88,9 +88,9 @@ typedef struct {
                         zero bias, more round-to-nearest additions, slower; 0 or -1 =
                         off (the default)                                                */
     int wait_limit_us; /* > 0: every bounded device wait of this handle's kernels (grid
-                        barriers of the solve, tensor-core pipeline barriers) gives up
-                        after this many microseconds; 0 = 1 s for the solve, 0.5 s for
-                        the pipeline.  On expiry the kernel records the error, drains
+                        barriers of the solve, pipeline barriers of the tensor-core and
+                        FP64 contractions) gives up after this many microseconds; 0 = 1 s
+                        for the solve, 0.5 s for the pipelines.  On expiry the kernel records the error, drains
                         what it issued and returns; the call reports PPL_ETIMEOUT.     */
     int acc_steps_p; /* as acc_steps, for the contractions of the S-build (W_b, S, P, and
                         W_a, which it then forms itself instead of taking the mode-b
@@ -317,6 +317,13 @@ int ppl_cp_energy_static(int o, int v, int X, int R, const double* B, const doub
  * usable; the factors are left mid-update, so reset them
  * (ppl_cpd_factors_changed) before further sweeps.  Works under graph replay. */
 int ppl_cpd_inject_wait_timeout(ppl_cpd* h);
+
+/* The same for the waits of the FP64 contractions by digit products: in the next such
+ * contraction of the handle (every contraction of an FP64 handle with K >= 8; energy,
+ * exact contraction, reconstruction and eta of the others) the first stage of one block
+ * never fills.  Its waits run out after opts.wait_limit_us (or 0.5 s), and the call that
+ * reads the result reports PPL_ETIMEOUT. */
+int ppl_cpd_inject_contraction_timeout(ppl_cpd* h);
 
 /* Measured FP64 FMA throughput of the current device (no counterpart in the
  * paper; the peak of the FP64 roofline the benchmark reports the solves

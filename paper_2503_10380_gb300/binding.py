@@ -90,6 +90,7 @@ def lib() -> ctypes.CDLL:
                                        c_void_p]
     L.ppl_cp_energy_static.restype = c_int
     L.ppl_cpd_inject_wait_timeout.argtypes = [H]
+    L.ppl_cpd_inject_contraction_timeout.argtypes = [H]
     L.ppl_probe_fp64_peak.argtypes = [POINTER(c_double), c_void_p]
     L.ppl_test_reciprocal.argtypes = [c_void_p, c_void_p, c_int, c_void_p]
     for name in ("ppl_cpd_workspace_size", "ppl_cpd_init", "ppl_cpd_mttkrp", "ppl_cpd_sweep",
@@ -99,6 +100,7 @@ def lib() -> ctypes.CDLL:
                  "ppl_cpd_set_t1", "ppl_exact_contract_mixed",
                  "ppl_cpd_batch_create", "ppl_cpd_batch_sweep", "ppl_cpd_batch_destroy", "ppl_cpd_batch_kernels",
                  "ppl_tc_gemm_workspace_size", "ppl_tc_gemm", "ppl_cpd_inject_wait_timeout",
+                 "ppl_cpd_inject_contraction_timeout",
                  "ppl_probe_fp64_peak", "ppl_test_reciprocal"):
         getattr(L, name).restype = c_int
     _lib = L
@@ -287,6 +289,10 @@ def ppl_cpd_phase_ms(h) -> dict:
 
 def ppl_cpd_inject_wait_timeout(h):
     _check(lib().ppl_cpd_inject_wait_timeout(h), h)
+
+
+def ppl_cpd_inject_contraction_timeout(h):
+    _check(lib().ppl_cpd_inject_contraction_timeout(h), h)
 
 
 def ppl_probe_fp64_peak(stream_ptr=None) -> float:

@@ -266,6 +266,7 @@ struct ppl_cpd {
     unsigned long long* nclamp() const { return at<unsigned long long>(L.flags); }
     unsigned int* errflag() const { return reinterpret_cast<unsigned int*>(ws + L.flags + 8); }
     unsigned int* withhold() const { return reinterpret_cast<unsigned int*>(ws + L.flags + 48); }
+    unsigned int* starve() const { return reinterpret_cast<unsigned int*>(ws + L.flags + 52); }
     int dim(int m) const { return m < 2 ? v : o; }
     bool tc() const { return opts.precision != PPL_PREC_FP64; }
     // bytes of one operand element over all its planes
@@ -444,6 +445,8 @@ void gemm(ppl_cpd* h, G64& g, bool operand = false) {
     g.err = h->errflag();
     g.scratch = h->at<unsigned long long>(h->L.rowx);
     g.nscratch = h->L.nrowx;
+    g.wait_ns = h->wait_ns;
+    g.withhold = h->starve();
     gemm64(g, h->st);
 }
 
@@ -1596,19 +1599,28 @@ int ppl_cpd_stats_get(ppl_cpd* h, ppl_cpd_stats* s) {
 
 const char* ppl_last_error(const ppl_cpd* h) { return h ? h->err.c_str() : g_err.c_str(); }
 
-int ppl_cpd_inject_wait_timeout(ppl_cpd* h) {
-    if (!h) return fail(nullptr, PPL_EINVAL, "NULL handle");
+static int arm(ppl_cpd* h, unsigned int* flag, const char* what) {
     int e = enter(h);
     if (e) return e;
     const unsigned int one = 1u;
-    cudaMemcpyAsync(h->withhold(), &one, sizeof one, cudaMemcpyHostToDevice, h->st);
-    e = check_cuda(h, "inject_wait_timeout");
+    cudaMemcpyAsync(flag, &one, sizeof one, cudaMemcpyHostToDevice, h->st);
+    e = check_cuda(h, what);
     if (!e) {
         const cudaError_t ce = cudaStreamSynchronize(h->st);
-        if (ce != cudaSuccess) e = fail(h, PPL_ECUDA, "inject_wait_timeout: %s", cudaGetErrorString(ce));
+        if (ce != cudaSuccess) e = fail(h, PPL_ECUDA, "%s: %s", what, cudaGetErrorString(ce));
     }
     leave(h);
     return e;
+}
+
+int ppl_cpd_inject_wait_timeout(ppl_cpd* h) {
+    if (!h) return fail(nullptr, PPL_EINVAL, "NULL handle");
+    return arm(h, h->withhold(), "inject_wait_timeout");
+}
+
+int ppl_cpd_inject_contraction_timeout(ppl_cpd* h) {
+    if (!h) return fail(nullptr, PPL_EINVAL, "NULL handle");
+    return arm(h, h->starve(), "inject_contraction_timeout");
 }
 
 }  // extern "C"

@@ -30,6 +30,8 @@ struct G64 {
     unsigned int* err;
     unsigned long long* scratch;
     long long nscratch;
+    unsigned long long wait_ns;   // limit of each wait (0: half a second)
+    unsigned int* withhold;       // test of the waits: != 0 makes one of the first block's run out (once)
 };
 void gemm64(const G64& g, cudaStream_t s);
 // the same on the tensor cores by exact digit products (ppl_split64.cu), with g.err and

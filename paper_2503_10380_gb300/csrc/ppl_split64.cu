@@ -355,7 +355,11 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
         s_bad = 0;
         s_zeros = 0;
         s_empty = 0;
-        mbar_init(full0, EWORK / 32);
+        // the test of the bounded waits: one arrival more than there are warps, so that the
+        // first stage never fills and every wait behind it runs out
+        const bool starve = blockIdx.x == 0 && blockIdx.z == 0 && g.withhold && *(volatile unsigned int*)g.withhold != 0u &&
+                            atomicExch(g.withhold, 0u) != 0u;
+        mbar_init(full0, EWORK / 32 + (starve ? 1 : 0));
         mbar_init(full0 + 8, EWORK / 32);
         mbar_init(bar0, 1);
         mbar_init(bar0 + 8, 1);
@@ -390,7 +394,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
 
     volatile int* vfail = &s_fail;
     // wait for the MMAs of k block kb
-    auto done = [&](int kb) { return mbar_wait(bar0 + 8u * (kb & 1), (uint32_t)(kb >> 1) & 1u, EWAIT_NS); };
+    auto done = [&](int kb) { return mbar_wait(bar0 + 8u * (kb & 1), (uint32_t)(kb >> 1) & 1u, g.wait_ns); };
     if (warp >= EWORK / 32) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(EREG_CTRL) : "memory");
         if (warp != EWORK / 32) return;
@@ -398,8 +402,8 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_gemm64_split(const __grid_const
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)EN >> 3 << 17) | ((uint32_t)(EM >> 4) << 24);
             int kb = 0;
             for (; kb < nkb && !*vfail; ++kb) {
-                if ((kb > 0 && kb % FOLD == 0 && !mbar_wait(folded, (uint32_t)(kb / FOLD - 1) & 1u, EWAIT_NS)) ||
-                    !mbar_wait(full0 + 8u * (kb & 1), (uint32_t)(kb >> 1) & 1u, EWAIT_NS)) {
+                if ((kb > 0 && kb % FOLD == 0 && !mbar_wait(folded, (uint32_t)(kb / FOLD - 1) & 1u, g.wait_ns)) ||
+                    !mbar_wait(full0 + 8u * (kb & 1), (uint32_t)(kb >> 1) & 1u, g.wait_ns)) {
                     *vfail = 1;
                     break;
                 }
@@ -728,6 +732,7 @@ int gemm64_split(const G64& g, cudaStream_t s) {
     if (tiles > 0x7fffffffll || z > 65535 || g.K / g.ksplit >= (1 << 24)) return -2;
     SplitArgs a;
     a.g = g;
+    if (a.g.wait_ns == 0) a.g.wait_ns = EWAIT_NS;
     a.ba = g.ab != 0;
     a.bb = g.bb != 0;
     const long long na = (long long)g.M * (a.ba ? g.batch : 1) * g.ksplit, nb = (long long)g.N * (a.bb ? g.batch : 1) * g.ksplit;

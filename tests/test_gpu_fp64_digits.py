@@ -14,6 +14,7 @@ be tried:
 """
 
 import math
+import time
 from fractions import Fraction
 
 import numpy as np
@@ -34,14 +35,14 @@ def _lib():
     __graft_entry__.build()
 
 
-def _handle(A, B, precision="fp64"):
+def _handle(A, B, precision="fp64", **opts):
     """A handle whose reconstruction is A B^T: A [v][K] in mode a, B [o][K] in mode i."""
     (v, K), o = A.shape, B.shape[0]
     fac = {"a": A, "b": np.ones((v, K)), "i": B, "j": np.ones((o, K))}
     g = torch.Generator().manual_seed(0)
     Bt = torch.randn(2, o + v, o + v, generator=g, dtype=torch.float64)
     tau = torch.randn(o, o, v, v, generator=g, dtype=torch.float64)
-    return binding.CpAls((Bt + Bt.transpose(1, 2)).cuda(), tau.cuda(), fac, precision=precision)
+    return binding.CpAls((Bt + Bt.transpose(1, 2)).cuda(), tau.cuda(), fac, precision=precision, **opts)
 
 
 def _products(A, B, precision="fp64"):
@@ -177,3 +178,46 @@ def test_cost_of_rows_with_zeros():
         ms.append(best)
         cp.close()
     assert ms[1] <= 6.0 * ms[0], ms
+
+
+@pytest.mark.parametrize("precision", ["fp64", "tf32x3"])
+@pytest.mark.parametrize("K", [24, 300])
+def test_wait_limit_holds(precision, K):
+    """A wait that runs out (the first stage of one block never fills): the call reports
+    PPL_ETIMEOUT after the handle's limit of 20 ms, not the default of 500, the other
+    blocks' results stand aside, and the next call is right again."""
+    rng = np.random.default_rng(5)
+    A, B = 0.5 + rng.random((40, K)), 0.5 + rng.random((6, K))
+    cp = _handle(A, B, precision, wait_limit_us=20000)
+    before = cp.reconstruct(symmetrise=False)
+    binding.ppl_cpd_inject_contraction_timeout(cp.h)
+    t0 = time.perf_counter()
+    with pytest.raises(binding.PplError) as e:
+        cp.reconstruct(symmetrise=False)
+    elapsed = time.perf_counter() - t0
+    assert e.value.code == binding.PPL_ETIMEOUT, str(e.value)
+    assert 0.015 < elapsed < 0.4, elapsed
+    assert cp.stats()["timeouts"] == 1
+    assert torch.equal(cp.reconstruct(symmetrise=False), before)
+    assert cp.stats()["timeouts"] == 1
+    cp.close()
+
+
+def test_wait_limit_holds_in_a_captured_sweep():
+    rng = np.random.default_rng(6)
+    fac = {m: rng.standard_normal((24 if m in "ab" else 5, 16)) for m in "abij"}
+    cp = _handle(fac["a"], fac["i"], wait_limit_us=20000)
+    cp.set_factors(fac)
+    cp.sweep(1)                          # captured; the flag is read at run time
+    first = {m: x.clone() for m, x in cp.factors().items()}
+    cp.set_factors(fac)
+    binding.ppl_cpd_inject_contraction_timeout(cp.h)
+    with pytest.raises(binding.PplError) as e:
+        cp.sweep(1)
+    assert e.value.code == binding.PPL_ETIMEOUT, str(e.value)
+    cp.set_factors(fac)
+    cp.sweep(1)
+    for m, x in cp.factors().items():
+        assert torch.allclose(x, first[m], rtol=1e-9, atol=1e-9 * float(first[m].abs().max()))
+    assert cp.stats()["timeouts"] == 1
+    cp.close()
