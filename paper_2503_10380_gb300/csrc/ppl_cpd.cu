@@ -1077,6 +1077,9 @@ int ppl_cpd_init(ppl_cpd** hp, int o, int v, int X, int R, const double* B, cons
         return fail(nullptr, PPL_ENOMEM, "workspace has %zu bytes, needs %zu", ws_bytes, L.total);
     if (op.precision != PPL_PREC_FP64 && tc_init_driver() != 0)
         return fail(nullptr, PPL_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
+    // (never a silent way back to the CUDA cores, 5 to 25 times slower)
+    if (const int r = gemm64_split_init())
+        return fail(nullptr, PPL_ECUDA, "the FP64 contraction kernel cannot run as it was built (%d)", r);
     ppl_cpd* h = new (std::nothrow) ppl_cpd();
     if (!h) return fail(nullptr, PPL_EINVAL, "out of host memory");
     h->o = o; h->v = v; h->X = X; h->R = R; h->n = o + v;

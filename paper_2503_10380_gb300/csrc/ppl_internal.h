@@ -37,6 +37,9 @@ void gemm64(const G64& g, cudaStream_t s);
 // the same on the tensor cores by exact digit products (ppl_split64.cu), with g.err and
 // g.scratch; nonzero (nothing launched) where the shape is out of its range
 int gemm64_split(const G64& g, cudaStream_t s);
+// once per handle, for the current device: shared memory opt-in and the register check of
+// the kernel; nonzero when it cannot run as built
+int gemm64_split_init();
 // from this K on: a k block of 32 costs 8k clocks however few are used, the CUDA cores 2k per k and tile
 constexpr int SPLIT64_MIN_K = 8;
 

@@ -48,7 +48,7 @@ constexpr int EWORK = 512;                     // threads that extract digits an
 constexpr int ETHREADS = EWORK + 128;          // and a warpgroup of which warp 16 issues the MMAs
 // Registers: 96 per thread at launch; the control warpgroup hands some to the workers
 // (88-bit sums of 16 columns each): 128 * 64 + 512 * 104 = 640 * 96 (checked on the host
-// before the first launch: a split above the launch's allocation would wait forever).
+// when a handle is made: a split above the launch's allocation would wait forever).
 // Sixteen working warps, not eight with twice the sums: the digit extraction is a
 // stream of dependent integer instructions.
 constexpr int EREG_LAUNCH = 96, EREG_CTRL = 64, EREG_WORK = 104;
@@ -710,21 +710,17 @@ RowArgs row_args(const double* p, const Idx2& rm, const Idx2& km, long long bs, 
 
 }  // namespace
 
-int gemm64_split(const G64& g, cudaStream_t s) {
-    static bool attr = false;
-    if (!attr) {
-        if (cudaFuncSetAttribute(k_gemm64_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ESMEM) != cudaSuccess) {
-            cudaGetLastError();
-            return -1;
-        }
-        cudaFuncAttributes fa;
-        if (cudaFuncGetAttributes(&fa, k_gemm64_split) != cudaSuccess) {
-            cudaGetLastError();
-            return -1;
-        }
-        if (fa.numRegs != EREG_LAUNCH || fa.maxThreadsPerBlock < ETHREADS) return -3;
-        attr = true;
+int gemm64_split_init() {
+    cudaFuncAttributes fa;
+    if (cudaFuncSetAttribute(k_gemm64_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ESMEM) != cudaSuccess ||
+        cudaFuncGetAttributes(&fa, k_gemm64_split) != cudaSuccess) {
+        cudaGetLastError();
+        return -1;
     }
+    return fa.numRegs == EREG_LAUNCH && fa.maxThreadsPerBlock >= ETHREADS ? 0 : -2;
+}
+
+int gemm64_split(const G64& g, cudaStream_t s) {
     if (g.lower) return -5;        // (Gram matrices of the CUDA-core form only)
     const long long tiles = (long long)((g.M + EM - 1) / EM) * ((g.N + EN - 1) / EN);
     const long long z = (long long)g.batch * g.ksplit;
