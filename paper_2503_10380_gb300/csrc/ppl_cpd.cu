@@ -32,6 +32,13 @@ thread_local std::string g_err;
 
 long long rup(long long x, long long m) { return (x + m - 1) / m * m; }
 
+// Room for the row statistics of an FP64 contraction, eight bytes per operand row, in a
+// part of the workspace that the call does not use otherwise.
+struct Rows {
+    size_t at;
+    long long n;
+};
+
 struct Layout {
     // offsets (bytes) into the workspace; -1 = absent
     size_t G[4], V, Linv, Z, M, P, scal, partial, hist, flags, KR64, Uold[4], lamold, Xc[4];
@@ -42,11 +49,15 @@ struct Layout {
     size_t Za, Zb, gov, Gblk, Rblk;
     size_t ring, cache, guess0;   // 6 iterates, the Near-Optimal cache, the initial guess
     size_t recon;                 // Khatri-Rao chunks for the reconstruction
-    size_t rowx;                  // eight bytes per operand row of an FP64 contraction
-    long long nrowx;
+    Rows rows, rows_exact, rows_recon;   // of sweeps, MTTKRPs, energy; exact contractions; reconstruction
+    size_t kr;                    // Khatri-Rao chunks of the reconstruction, rcr columns
     int rcr;
+    // tensor-core exact contraction of ng > 1 rows a per launch: G in Gblk, the split-K
+    // partials of R at Gpart, of which part_dirty bytes overlay sweep intermediates
+    size_t Gpart, part_dirty;
     size_t total;
-    int rc, na, ng;               // r-chunk; rows a per launch of the exact contraction, FP64 and tensor-core
+    int rc, na;                   // r-chunk; rows a per launch of the exact contraction
+    int ng, nr;                   // rows a per launch of the tensor-core one: G, R
     long long ldv, ldX, ldo2, ldvv;
     long long ldk;   // tensor-core form: v padded to the K-panel width (a K extent of v per block of a compound index)
     int ke;          // the K-panel width: elements of one 128-byte operand row
@@ -54,10 +65,6 @@ struct Layout {
 
 constexpr int NPART = 2 * 304 + 8;
 constexpr int KSMAX = 80;   // most split-K slices of one tensor-core contraction
-// Bound of G of the rows a that one launch of the tensor-core exact contraction takes (the
-// FP64 form's block of G, in which the partials of the mixed form lie, is as large).
-// At o 14, v 120, X 360: 64 MB 3.63 ms, 128 MB 2.83, 256 MB 2.42, one row per launch 7.29.
-constexpr size_t EXACT_BYTES = (size_t)256 << 20;
 constexpr int RC_MAX = 1024; // most rank columns per pass of the chain
 #ifndef TF32X3_ACC_STEPS
 #define TF32X3_ACC_STEPS 0      // default MMA K steps per TF32X3 accumulation chunk (0: a K block)
@@ -141,24 +148,26 @@ bool plan(int o, int v, int X, int R, const ppl_cpd_opts& op, Layout& L) {
     L.gov = take((size_t)o * v * o * v * d);
     L.Gblk = take((size_t)na * v3 * d);
     L.Rblk = take((size_t)na * v * o * o * d);
+    const long long nvo = (long long)v * v + (long long)o * o;
+    L.recon = take((size_t)nvo * (R < 64 ? R : 64) * d);
+    // gov .. recon are idle in sweeps, MTTKRPs and energies, which keep the statistics of
+    // their operand rows there (a pair of operands with more rows than fit is contracted on
+    // the CUDA cores; up to X = 6 v and R = 8 v that is Y, W and the energy below v = 8,
+    // whose K = v is too short for the digits as well).
+    L.rows = {L.gov, (long long)((off - L.gov) / sizeof(unsigned long long))};
+    // A reconstruction uses none of KR64 .. recon otherwise: its nvo rows first, then
+    // Khatri-Rao chunks of up to 256 columns (each chunk is a pass over R~, and a rounding).
+    L.rows_recon = {L.KR64, nvo};
+    L.kr = L.KR64 + (size_t)rup(nvo * (long long)sizeof(unsigned long long), 256);
+    long long rcr = (long long)((off - L.kr) / d) / nvo;
+    if (rcr > 256) rcr = 256;
+    L.rcr = (int)(rcr < R ? rcr : R);
+    // an exact contraction leaves the Khatri-Rao chunks alone, and the intermediates below
+    L.rows_exact = {L.recon, (long long)((off - L.recon) / sizeof(unsigned long long))};
     const size_t fsz = (size_t)(2 * v + 2 * o + 1) * R * d;
     L.ring = take(6 * fsz);
     L.cache = take(fsz);
     L.guess0 = take(fsz);
-    L.rcr = R < 256 ? R : 256;
-    L.recon = take((size_t)((long long)v * v + (long long)o * o) * L.rcr * d);
-    // the widest pair of operands: W or the dressing (X v and rc or v rows), Y or S (per
-    // batch entry), the energy, the exact contraction, the reconstruction, a Gram matrix
-    {
-        const long long xv = (long long)X * v, vv = (long long)v * v, oo = (long long)o * o;
-        const long long pairs[] = {xv + v + rc, (long long)rc * ((long long)X + 2 * v), (long long)X * o + R, vv + oo + R,
-                                   na * v + vv + oo, 2ll * o * v, 2ll * R,
-                                   // split over K: M and P of the FP64 form, up to FP64_KSPLIT slices
-                                   (long long)FP64_KSPLIT * (v + rc), (long long)FP64_KSPLIT * (oo + rc)};
-        L.nrowx = 0;
-        for (long long n : pairs) L.nrowx = n > L.nrowx ? n : L.nrowx;
-        L.rowx = take((size_t)L.nrowx * sizeof(unsigned long long));
-    }
     const size_t none = (size_t)-1;
     L.T64 = L.W64 = L.Y64 = L.S64 = none;
     L.tauT = L.tauN = L.Bn = L.Bp = L.BpW = L.UopA = L.UopB = L.KRT = L.T = L.Tt = L.W = L.Y = L.WTa = L.WTb = L.S = none;
@@ -167,13 +176,17 @@ bool plan(int o, int v, int X, int R, const ppl_cpd_opts& op, Layout& L) {
     L.PART = none;
     L.Bbar = L.BbN = L.BbP = L.BbT = none;
     L.Bq = L.BbQ = L.Gop = none;
-    L.ng = 0;
+    L.ng = L.nr = 0;
+    L.Gpart = none;
+    L.part_dirty = 0;
     if (op.dressed) L.Bbar = take((size_t)X * v * v * d);
     if (!tc) {
         L.T64 = take((size_t)R * v * v * d);
         L.W64 = take((size_t)rc * X * v * d);
         L.Y64 = take((size_t)rc * X * v * d);
         L.S64 = take((size_t)rc * v * v * d);
+        const long long nx = (long long)((off - L.T64) / sizeof(unsigned long long));
+        if (nx > L.rows_exact.n) L.rows_exact = {L.T64, nx};
     } else {
         // operands in the K-panel layout (rows x K, K padded to the panel width ke)
         const size_t e = op.precision == PPL_PREC_TF32X3 ? 8 : 4;   // bf16 hi + lo, fp32 hi + lo, or one fp32
@@ -199,19 +212,32 @@ bool plan(int o, int v, int X, int R, const ppl_cpd_opts& op, Layout& L) {
         L.S = take((size_t)rc * kvv * e);                  // rows r, K = (c, d)
         {
             const size_t chain_part = (size_t)KSMAX * (size_t)(v > o * o ? v : o * o) * rc;
-            // rows a of the exact contraction per launch: their G within EXACT_BYTES, the
-            // split-K partials of more than one within the FP64 form's block of G
-            const size_t part1 = (size_t)KSMAX * (size_t)v * o * o * sizeof(float);
-            long long ng = (long long)(EXACT_BYTES / ((size_t)v * kvv * e));
-            const long long np = (long long)((size_t)na * v3 * d / part1);
-            if (ng > np) ng = np;
-            if (ng > na) ng = na;
-            L.ng = ng < 1 ? 1 : (int)ng;
+            const size_t part1 = (size_t)KSMAX * (size_t)v * o * o * sizeof(float), g1 = (size_t)v * kvv * e;
             const size_t exact_part = part1 / sizeof(float);
             L.PART = take((chain_part > exact_part ? chain_part : exact_part) * sizeof(float));
+            const long long nx = (long long)((off - L.PART) / sizeof(unsigned long long));
+            if (nx > L.rows_exact.n) L.rows_exact = {L.PART, nx};
+            // Rows a of the exact contraction per launch of G, ng, and of R, nr (both equal, o 14,
+            // v 120, X 360: one 7.29 ms, four 3.63, nine 2.83, seventeen 2.42): G in the FP64
+            // form's block of G; the partials of R at the end of the sweep's intermediates T ..
+            // PART, or behind G where that takes more rows.
+            const size_t blk = L.Rblk - L.Gblk;
+            const long long gmax = (long long)(blk / g1), over = (long long)((off - L.T) / part1);
+            const long long behind = (long long)(blk / (g1 + part1));
+            const bool at_end = (over < gmax ? over : gmax) >= behind;
+            const long long ng = at_end ? gmax : behind;
+            L.ng = (int)(ng < na ? ng : na);
+            if (L.ng > 1) {
+                const long long passes = at_end ? (L.ng + over - 1) / over : 1;
+                L.nr = (int)((L.ng + passes - 1) / passes);
+                L.Gpart = at_end ? (off - L.nr * part1) / 256 * 256 : L.Gblk + L.ng * g1;
+                L.part_dirty = at_end && L.Gpart < L.PART ? L.PART - L.Gpart : 0;
+            } else {
+                L.ng = L.nr = 1;
+            }
         }
         L.Bq = take(vv * kX * e);                          // rows (p,q), K = Q
-        L.Gop = take((size_t)L.ng * v * kvv * e);          // per a: rows b, K = (c, d)
+        L.Gop = take((size_t)v * kvv * e);                 // rows b, K = (c, d), of one row a
         if (op.dressed) L.BbQ = take(vv * kX * e);
         if (op.dressed) {
             L.BbN = take(Xv * L.ldk * e);
@@ -437,14 +463,14 @@ int run_tc(ppl_cpd* h, TcGemm& g, const char* what) {
 // matters: at a rounding boundary of an operand it moves every later sweep by the
 // split precision's noise, so the tensor-core forms sum those on the CUDA cores, in
 // the order of k; nothing else does.
-void gemm(ppl_cpd* h, G64& g, bool operand = false) {
+void gemm(ppl_cpd* h, G64& g, const Rows& rows, bool operand = false) {
     if (operand && h->tc()) {
         gemm64(g, h->st);
         return;
     }
     g.err = h->errflag();
-    g.scratch = h->at<unsigned long long>(h->L.rowx);
-    g.nscratch = h->L.nrowx;
+    g.scratch = h->at<unsigned long long>(rows.at);
+    g.nscratch = rows.n;
     g.wait_ns = h->wait_ns;
     g.withhold = h->starve();
     gemm64(g, h->st);
@@ -458,7 +484,7 @@ void gram(ppl_cpd* h, int m) {
     g.C = h->G(m); g.cm = ix1(R); g.cn = ix1(1);
     g.M = R; g.N = R; g.K = h->dim(m); g.batch = 1; g.ksplit = 1; g.alpha = 1.0;
     g.lower = h->tc();     // symmetric: half the FP64 work
-    gemm(h, g, true);
+    gemm(h, g, h->L.rows, true);
 }
 
 // the arguments of mode m's update: V from the other three Gram matrices, M from L.M
@@ -501,7 +527,7 @@ void t_fp64(ppl_cpd* h) {
     g.B = h->tau; g.bn = ix1(1); g.bk = ix1((long long)v * v);
     g.C = h->at<double>(h->L.T64); g.cm = ix1((long long)v * v); g.cn = ix1(1);
     g.M = R; g.N = v * v; g.K = o * o; g.batch = 1; g.ksplit = 1; g.alpha = 1.0;
-    gemm(h, g);
+    gemm(h, g, h->L.rows);
 }
 
 // W[r][Q][d] = sum_b B[Q][o+b][o+d] U[b][r0+r]; bside: the dressed D-bar[Q][b][d]
@@ -516,7 +542,7 @@ void w_fp64(ppl_cpd* h, const double* U, int r0, int rcur, double* W, bool bside
     g.B = U + r0; g.bn = ix1(1); g.bk = ix1(R);
     g.C = W; g.cm = ix1(1); g.cn = ix1((long long)X * v);
     g.M = X * v; g.N = rcur; g.K = v; g.batch = 1; g.ksplit = 1; g.alpha = 1.0;
-    gemm(h, g);
+    gemm(h, g, h->L.rows);
 }
 
 void mttkrp_ab_fp64(ppl_cpd* h, int mode, double* Mout) {
@@ -535,7 +561,7 @@ void mttkrp_ab_fp64(ppl_cpd* h, int mode, double* Mout) {
         else           { y.bn = ix1(1); y.bk = ix1(v); }   // T[r][c][d], contract c
         y.C = Y; y.cb = (long long)X * v; y.cm = ix1(v); y.cn = ix1(1);
         y.M = X; y.N = v; y.K = v; y.batch = rcur; y.ksplit = 1; y.alpha = 1.0;
-        gemm(h, y);
+        gemm(h, y, h->L.rows);
         G64 m{};
         if (mode == 1 && h->dressed()) {
             m.A = h->at<double>(h->L.Bbar); m.am = ix1(v); m.ak = ix2(v, (long long)v * v, 1);
@@ -549,7 +575,7 @@ void mttkrp_ab_fp64(ppl_cpd* h, int mode, double* Mout) {
         long long ks = (FP64_KSPLIT + tiles - 1) / tiles;
         if (ks > (X * (long long)v) / 64) ks = (X * (long long)v) / 64;
         m.ksplit = ks < 1 ? 1 : (int)ks;
-        gemm(h, m);
+        gemm(h, m, h->L.rows);
     }
 }
 
@@ -569,7 +595,7 @@ void p_fp64(ppl_cpd* h) {
         s.B = Wb; s.bb = (long long)X * v; s.bn = ix1(1); s.bk = ix1(v);
         s.C = S; s.cb = (long long)v * v; s.cm = ix1(v); s.cn = ix1(1);
         s.M = v; s.N = v; s.K = X; s.batch = rcur; s.ksplit = 1; s.alpha = 1.0;
-        gemm(h, s);
+        gemm(h, s, h->L.rows);
         G64 p{};
         p.A = h->tau; p.am = ix1((long long)v * v); p.ak = ix1(1);
         p.B = S; p.bn = ix1((long long)v * v); p.bk = ix1(1);
@@ -579,7 +605,7 @@ void p_fp64(ppl_cpd* h) {
         long long ks = (FP64_KSPLIT + tiles - 1) / tiles;
         if (ks > (long long)v * v / 64) ks = (long long)v * v / 64;
         p.ksplit = ks < 1 ? 1 : (int)ks;
-        gemm(h, p);
+        gemm(h, p, h->L.rows);
     }
 }
 
@@ -821,7 +847,7 @@ void build_dbar(ppl_cpd* h, const double* t1) {
         g.B = t1; g.bn = ix1(1); g.bk = ix1(v);                                            // t1[k][d]
         g.C = Bb; g.cb = (long long)v * v; g.cm = ix1(v); g.cn = ix1(1);
         g.M = v; g.N = v; g.K = o; g.batch = X; g.ksplit = 1; g.alpha = -2.0; g.beta = 1.0;
-        gemm(h, g, true);
+        gemm(h, g, h->L.rows, true);
     }
     if (!h->tc()) return;
     // D-bar[Q][b][d] is not symmetric in (b, d): the b side of every contraction reads it with b as the row index
@@ -868,7 +894,7 @@ int prepare_operands(ppl_cpd* h, bool tau_only) {
     zero_bytes(opb(h, h->L.WTa), (size_t)h->R * v * q.kX * eb, h->st);
     zero_bytes(opb(h, h->L.WTb), (size_t)h->L.rc * v * q.kX * eb, h->st);
     zero_bytes(opb(h, h->L.S), (size_t)h->L.rc * q.kvv * eb, h->st);
-    zero_bytes(opb(h, h->L.Gop), (size_t)h->L.ng * v * q.kvv * eb, h->st);
+    zero_bytes(opb(h, h->L.Gop), (size_t)v * q.kvv * eb, h->st);
     return PPL_OK;
 }
 
@@ -902,7 +928,7 @@ void cross_gram(ppl_cpd* h, int m) {
     g.B = h->at<double>(h->L.Uold[m]); g.bn = ix1(1); g.bk = ix1(R);
     g.C = h->at<double>(h->L.Xc[m]); g.cm = ix1(R); g.cn = ix1(1);
     g.M = R; g.N = R; g.K = h->dim(m); g.batch = 1; g.ksplit = 1; g.alpha = 1.0;
-    gemm(h, g);
+    gemm(h, g, h->L.rows);
 }
 
 // phase boundary; External makes the record a real event node when the
@@ -1263,7 +1289,7 @@ int ppl_cpd_energy(ppl_cpd* h, double* E_cp) {
         g.B = h->U[w]; g.bn = ix1(1); g.bk = ix1(R);
         g.C = Z[w]; g.cm = ix1(R); g.cn = ix1(1);
         g.M = X * o; g.N = R; g.K = v; g.batch = 1; g.ksplit = 1; g.alpha = 1.0;
-        gemm(h, g);
+        gemm(h, g, h->L.rows);
     }
     energy_reduce(Z[0], Z[1], h->U[2], h->U[3], h->lam, X, o, R, h->at<double>(h->L.partial),
                   h->scal() + SC_ENERGY, h->st);
@@ -1290,7 +1316,7 @@ int ppl_exact_contract(ppl_cpd* h, double* normR2, double* E_exact, double* R_ou
     g.B = h->B + o; g.bn = ix2(v, n, 1); g.bk = ix1((long long)n * n);
     g.C = gov; g.cm = ix1((long long)o * v); g.cn = ix1(1);
     g.M = o * v; g.N = o * v; g.K = X; g.batch = 1; g.ksplit = 1; g.alpha = 1.0;
-    gemm(h, g);
+    gemm(h, g, h->L.rows_exact);
     const long long v3 = (long long)v * v * v, vo2 = (long long)v * o * o;
     for (int a0 = 0; a0 < v; a0 += na) {
         const int nb = (v - a0 < na) ? v - a0 : na;
@@ -1304,7 +1330,7 @@ int ppl_exact_contract(ppl_cpd* h, double* normR2, double* E_exact, double* R_ou
         }
         q.C = Gb; q.cb = v3; q.cm = ix1((long long)v * v); q.cn = ix1(1);
         q.M = v; q.N = v * v; q.K = X; q.batch = nb; q.ksplit = 1; q.alpha = 1.0;
-        gemm(h, q);
+        gemm(h, q, h->L.rows_exact);
         // R[a][b][ij] = sum_{c,d} G_a[c][b][d] tau[ij][c][d]
         double* Rdst = R_out ? R_out + (long long)a0 * vo2 : Rb;
         G64 r{};
@@ -1312,7 +1338,7 @@ int ppl_exact_contract(ppl_cpd* h, double* normR2, double* E_exact, double* R_ou
         r.B = h->tau; r.bb = 0; r.bn = ix1((long long)v * v); r.bk = ix1(1);
         r.C = Rdst; r.cb = vo2; r.cm = ix1((long long)o * o); r.cn = ix1(1);
         r.M = v; r.N = o * o; r.K = v * v; r.batch = nb; r.ksplit = 1; r.alpha = 1.0;
-        gemm(h, r);
+        gemm(h, r, h->L.rows_exact);
         exact_reduce(Rdst, a0, nb, v, o, gov, h->at<double>(h->L.partial), acc, h->st);
     }
     e = check_cuda(h, "exact_contract");
@@ -1332,7 +1358,7 @@ int ppl_cpd_reconstruct(ppl_cpd* h, double* R_out, int symmetrise) {
     const int o = h->o, v = h->v, R = h->R, rcr = h->L.rcr;
     int e = enter(h);
     if (e) return e;
-    double* Kab = h->at<double>(h->L.recon);
+    double* Kab = h->at<double>(h->L.kr);
     double* Kij = Kab + (size_t)v * v * rcr;
     for (int r0 = 0; r0 < R; r0 += rcr) {
         const int rc = (R - r0 < rcr) ? R - r0 : rcr;
@@ -1344,7 +1370,7 @@ int ppl_cpd_reconstruct(ppl_cpd* h, double* R_out, int symmetrise) {
         g.C = R_out; g.cm = ix1((long long)o * o); g.cn = ix1(1);
         g.M = v * v; g.N = o * o; g.K = rc; g.batch = 1; g.ksplit = 1;
         g.alpha = 1.0; g.beta = (r0 == 0) ? 0.0 : 1.0;
-        gemm(h, g);
+        gemm(h, g, h->L.rows_recon);
     }
     if (symmetrise) symmetrise_pairs(R_out, v, o, h->st);
     e = check_cuda(h, "reconstruct");
@@ -1368,13 +1394,16 @@ int ppl_exact_contract_mixed(ppl_cpd* h, double* normR2, double* E_exact, double
     g.B = h->B + o; g.bn = ix2(v, n, 1); g.bk = ix1((long long)n * n);
     g.C = gov; g.cm = ix1((long long)o * v); g.cn = ix1(1);
     g.M = o * v; g.N = o * v; g.K = X; g.batch = 1; g.ksplit = 1; g.alpha = 1.0;
-    gemm(h, g);
+    gemm(h, g, h->L.rows_exact);
     const Pan pq = pan_of(h);
     // ng rows a per launch: one row's five launches of 5 to 17 us each ended in a tail of
     // idle SMs and a gap
     const int ng = h->L.ng;
     const long long pQ = (long long)v * v * pq.kX, bG = (long long)v * pq.kvv, pG = bG * ng;
-    float* part = h->at<float>(ng > 1 ? h->L.Gblk : h->L.PART);
+    float* part = h->at<float>(ng > 1 ? h->L.Gpart : h->L.PART);
+    void* G = opb(h, ng > 1 ? h->L.Gblk : h->L.Gop);
+    if (ng > 1)      // (Gop's K padding is zero as it is)
+        zero_padding(h->opts.precision, G, pG, (long long)ng * v, v, v, pq.ldk, h->st);
     for (int a = 0; a < v && !e; a += ng) {
         const int nb = (v - a < ng) ? v - a : ng;
         // G_a[b][c][d] = sum_Q D-bar[Q][b][d] B[Q][a][c]; per a: rows b, K (c, d); m = b*v + d, n = (a, c)
@@ -1383,21 +1412,26 @@ int ppl_exact_contract_mixed(ppl_cpd* h, double* normR2, double* E_exact, double
         g1.B = pmat(opb(h, h->L.Bq), pQ, v * v, X, 1, (long long)v * v, 0);
         g1.b_row0 = a * v;
         g1.M = v * v; g1.N = nb * v; g1.K = X; g1.batch = 1; g1.ksplit = 1;
-        g1.out = out_map(opb(h, h->L.Gop), pG, 0, v, plain(pq.ke, pq.ke), kpan((long long)v * pq.ke),
+        g1.out = out_map(G, pG, 0, v, plain(pq.ke, pq.ke), kpan((long long)v * pq.ke),
                          pq.ldk * v);
         e = run_tc(h, g1, "exact G");
         if (e) break;
         // R[a][b][ij] = sum_{cd} G_a[b][cd] tau[ij][cd], split-K summed in FP64
         double* Rdst = R_out ? R_out + (long long)a * vo2 : h->at<double>(h->L.Rblk);
-        TcGemm g2{};
-        g2.A = pmat(opb(h, h->L.Gop), pG, v, (int)pq.kvv, nb, v, bG);
-        g2.a_bstep = 1;
-        g2.B = pmat(opb(h, h->L.tauN), (long long)o * o * pq.kvv, o * o, (int)pq.kvv, 1, (long long)o * o, 0);
-        g2.M = v; g2.N = o * o; g2.K = (int)pq.kvv; g2.batch = nb;
-        e = run_tc_partial(h, g2, part, Rdst, (long long)o * o, vo2, "exact R");
+        for (int b0 = 0; b0 < nb && !e; b0 += h->L.nr) {
+            TcGemm g2{};
+            g2.A = pmat(G, pG, v, (int)pq.kvv, nb, v, bG);
+            g2.a_b0 = b0;
+            g2.a_bstep = 1;
+            g2.B = pmat(opb(h, h->L.tauN), (long long)o * o * pq.kvv, o * o, (int)pq.kvv, 1, (long long)o * o, 0);
+            g2.M = v; g2.N = o * o; g2.K = (int)pq.kvv; g2.batch = (nb - b0 < h->L.nr) ? nb - b0 : h->L.nr;
+            e = run_tc_partial(h, g2, part, Rdst + b0 * vo2, (long long)o * o, vo2, "exact R");
+        }
         if (e) break;
         exact_reduce(Rdst, a, nb, v, o, gov, h->at<double>(h->L.partial), acc, h->st);
     }
+    // the intermediates' K padding reads as zero again
+    if (h->L.part_dirty) zero_bytes(part, h->L.part_dirty, h->st);
     if (!e) e = check_cuda(h, "exact_contract_mixed");
     if (!e) e = sync_and_check(h);
     double res[2] = {0, 0};

@@ -195,3 +195,7 @@ void transpose_panels(int prec, const void* src, void* dst, long long plane_s, l
 // elements of one 128-byte operand row (the K-panel width) of a precision
 int panel_width(int prec);
 void zero_bytes(void* p, size_t n, cudaStream_t s);
+// zero the K padding of operand planes whose K index is (c, d), d < cols padded to ld: the
+// last panel of each group (batch entry, c), `rows` rows of it
+void zero_padding(int prec, void* p, long long plane_elems, long long groups, int rows, int cols, long long ld,
+                  cudaStream_t s);

@@ -895,6 +895,18 @@ __global__ void __launch_bounds__(RPT) k_reduce_partials(const float* part, long
     out[(long long)blockIdx.y * ob + (long long)m * ldo + n] = s;
 }
 
+// The last npad columns of the last K panel (of ld columns) of each group.  Two planes of 17 x
+// 120 groups of 120 rows: 31 MB of sectors.
+template <class T>
+__global__ void k_zero_padding(T* p, long long plane, long long groups, int rows, int ke, int npad, long long ld,
+                               long long total) {
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
+        const int t = (int)(e % npad), b = (int)(e / npad % rows);
+        const long long g = e / npad / rows;          // (plane, group)
+        p[g / groups * plane + (g % groups * ld + ld - ke) * rows + (long long)b * ke + ke - npad + t] = T(0);
+    }
+}
+
 // Batched transpose of operand planes: dst[b][j][i] = src[b][i][j] for i, j < n
 // (row stride ld); 2-byte elements in two planes (BF16X3) or 4-byte in one (TF32).
 template <typename T, int PLANES>
@@ -1377,6 +1389,17 @@ void transpose_panels(int prec, const void* src, void* dst, long long plane_s, l
 
 void zero_bytes(void* p, size_t n, cudaStream_t s) {
     if (n) cudaMemsetAsync(p, 0, n, s);
+}
+
+void zero_padding(int prec, void* p, long long plane_elems, long long groups, int rows, int cols, long long ld,
+                  cudaStream_t s) {
+    const int ke = panel_width(prec), npad = (int)(ld - cols), planes = prec == PPL_PREC_TF32 ? 1 : 2;
+    const long long total = (long long)planes * groups * rows * npad;
+    if (total <= 0) return;
+    if (prec == PPL_PREC_BF16X3)
+        k_zero_padding<<<grid_for(total, 256), 256, 0, s>>>((unsigned short*)p, plane_elems, groups, rows, ke, npad, ld, total);
+    else
+        k_zero_padding<<<grid_for(total, 256), 256, 0, s>>>((unsigned int*)p, plane_elems, groups, rows, ke, npad, ld, total);
 }
 
 // ---- several captured contractions as one persistent launch ------------------
