@@ -74,7 +74,8 @@ constexpr int NPC = 4;                        // pieces per epilogue warp (a 128
 // more warps read it and write it out.
 // 16 warps: 128 * 56 + 256 * 168 + 128 * 120 = 512 * 128 registers.
 constexpr int HBN = 160;                      // widest N tile of the handed-over form
-constexpr int HKB = 8;                        // most K blocks of a handed-over contraction
+// most K blocks of a handed-over contraction (measured where the rule is applied)
+constexpr int hand_kb(int prec) { return prec == PPL_PREC_TF32X3 ? 8 : prec == PPL_PREC_TF32 ? 7 : 6; }
 constexpr int HPW = 16;                       // columns per piece of a summing warp
 constexpr int HNP = HBN / 2 / HPW;            // pieces per summing warp
 constexpr int NSTORE = 4;                     // storing warps, one per TMEM lane quarter
@@ -1251,10 +1252,16 @@ int tc_gemm(const TcGemm& g, unsigned int* err_flag, cudaStream_t s) {
     // is what the time goes to.  Split TF32, wide tiles -> handed over: 7 K blocks (v 200,
     // X 600, R 800) W 278 -> 242 us, Y 362 -> 359; 8 (251, 773, 605) W 418 -> 415, Y 439
     // -> 397.  From 13 on the narrower tiles' loads cost more: W 692 -> 721, Y 789 -> 864
-    // (400, 1000, 400), and at 19 W 2678 -> 2779, Y 2977 -> 3111 (600, 1800, 480).
+    // (400, 1000, 400), and at 19 W 2678 -> 2779, Y 2977 -> 3111 (600, 1800, 480).  Whole
+    // MTTKRPs of mode a at 8: 0.99 to 1.01 of the wide form's time over R 350 .. 1000.
+    // Restarted TF32 (half the stores): 7 blocks 0.96 .. 1.05 times as fast, 8 blocks (250,
+    // 750, 1000) 1294 -> 1393 us, (250, 375, 500) 518 -> 547.  Restarted BF16X3 (K blocks
+    // twice as long): 4 blocks (200, 600, 800) 813 -> 712, 5 blocks 1500 -> 1398, 6 blocks
+    // 2968 -> 2962 and 2654 -> 2520, 7 blocks (400, 1200, 1000) 4743 -> 4803, 8 blocks (500,
+    // 1500, 1000) 8520 -> 8635.
     // Split-K partials keep the wide tiles: their K is long.
     const bool drain = p.ksub > 0 || (g.kchunk > 0 && g.kchunk < p.per_split);
-    const int mode = !drain ? 0 : (g.out.kind == EPI_SPLIT && p.ksub == 0 && p.nkb_total <= HKB) ? 2 : 1;
+    const int mode = !drain ? 0 : (g.out.kind == EPI_SPLIT && p.ksub == 0 && p.nkb_total <= hand_kb(g.prec)) ? 2 : 1;
     if (mode == 2) {
         const int nt = (g.N + HBN - 1) / HBN;
         p.bn = ((g.N + nt - 1) / nt + 15) / 16 * 16;
