@@ -171,9 +171,8 @@ def test_short_restarted_sums_handed_over(prec, shape):
 @pytest.mark.parametrize("spread", [0, 12, 40, 80])
 @pytest.mark.parametrize("shape", [(5, 24, 72, 48), (3, 33, 97, 9)])
 def test_split_k_slices_of_mixed_magnitude(shape, spread):
-    """Split-K slices whose exponents lie up to 2 spread apart: the sum over slices as
-    integers, the FP64 loop beyond its range, and elements on both sides of it in one
-    tile.  Column r of the result has its own scale, so the chain bound and the
+    """Split-K slices whose exponents lie up to 2 spread apart, all within FP32's normal
+    numbers.  Column r of the result has its own scale, so the chain bound and the
     per-column bound hold as they do without the scaling."""
     o, v, X, R = shape
     inp = inputs.make_inputs(o, v, X, R, seed=4)
@@ -211,7 +210,7 @@ def test_solve_at_block_edges(R):
     """The solve's 32-wide blocks at their edges (a last block of 1, 2, 31 or 32
     columns, one to six blocks): FP64 sweeps against the oracle, with the clamped
     pivots counted alike (R = 161 exceeds the rank 10 * 4 * 4 of V for modes a and
-    b, so it is singular there and only the first sweep's count is compared)."""
+    b, so it is singular there: one sweep, which clamps and stays finite)."""
     o, v, X = 4, 10, 12
     inp = inputs.make_inputs(o, v, X, R, seed=13)
     cp = binding.CpAls(_dev(inp.B), _dev(inp.tau), inp.factors, precision="fp64")
