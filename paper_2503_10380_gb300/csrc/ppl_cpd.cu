@@ -52,7 +52,7 @@ struct Layout {
     Rows rows, rows_exact, rows_recon;   // of sweeps, MTTKRPs, energy; exact contractions; reconstruction
     size_t kr;                    // Khatri-Rao chunks of the reconstruction, rcr columns
     int rcr;
-    // tensor-core exact contraction of ng > 1 rows a per launch: G in Gblk, the split-K
+    // tensor-core exact contraction of ng > 1 rows a per launch: G at KR64, the split-K
     // partials of R at Gpart, of which part_dirty bytes overlay sweep intermediates
     size_t Gpart, part_dirty;
     size_t total;
@@ -139,22 +139,22 @@ bool plan(int o, int v, int X, int R, const ppl_cpd_opts& op, Layout& L) {
     L.partial = take(NPART * d);
     L.hist = take(4 * d);
     L.flags = take(64);
+    L.gov = take((size_t)o * v * o * v * d);
     L.KR64 = take((size_t)R * o * o * d);
     for (int m = 0; m < 4; ++m) L.Uold[m] = take((size_t)dim * R * d);
     L.lamold = take((size_t)R * d);
     for (int m = 0; m < 4; ++m) L.Xc[m] = take(RR * d);
     L.Za = take((size_t)X * o * R * d);
     L.Zb = take((size_t)X * o * R * d);
-    L.gov = take((size_t)o * v * o * v * d);
     L.Gblk = take((size_t)na * v3 * d);
     L.Rblk = take((size_t)na * v * o * o * d);
     const long long nvo = (long long)v * v + (long long)o * o;
     L.recon = take((size_t)nvo * (R < 64 ? R : 64) * d);
-    // gov .. recon are idle in sweeps, MTTKRPs and energies, which keep the statistics of
+    // Gblk .. recon are idle in sweeps, MTTKRPs and energies, which keep the statistics of
     // their operand rows there (a pair of operands with more rows than fit is contracted on
     // the CUDA cores; up to X = 6 v and R = 8 v that is Y, W and the energy below v = 8,
     // whose K = v is too short for the digits as well).
-    L.rows = {L.gov, (long long)((off - L.gov) / sizeof(unsigned long long))};
+    L.rows = {L.Gblk, (long long)((off - L.Gblk) / sizeof(unsigned long long))};
     // A reconstruction uses none of KR64 .. recon otherwise: its nvo rows first, then
     // Khatri-Rao chunks of up to 256 columns (each chunk is a pass over R~, and a rounding).
     L.rows_recon = {L.KR64, nvo};
@@ -218,19 +218,21 @@ bool plan(int o, int v, int X, int R, const ppl_cpd_opts& op, Layout& L) {
             const long long nx = (long long)((off - L.PART) / sizeof(unsigned long long));
             if (nx > L.rows_exact.n) L.rows_exact = {L.PART, nx};
             // Rows a of the exact contraction per launch of G, ng, and of R, nr (both equal, o 14,
-            // v 120, X 360: one 7.29 ms, four 3.63, nine 2.83, seventeen 2.42): G in the FP64
-            // form's block of G; the partials of R at the end of the sweep's intermediates T ..
-            // PART, or behind G where that takes more rows.
-            const size_t blk = L.Rblk - L.Gblk;
+            // v 120, X 360: one 7.29 ms, four 3.63, nine 2.83, seventeen 2.42): G in KR64 .. Gblk,
+            // which only other calls use; the partials of R at the end of the sweep's
+            // intermediates T .. PART, or behind G where that takes more rows.
+            const size_t blk = L.Rblk - L.KR64;
             const long long gmax = (long long)(blk / g1), over = (long long)((off - L.T) / part1);
             const long long behind = (long long)(blk / (g1 + part1));
             const bool at_end = (over < gmax ? over : gmax) >= behind;
-            const long long ng = at_end ? gmax : behind;
-            L.ng = (int)(ng < na ? ng : na);
+            long long ng = at_end ? gmax : behind;
+            if (ng > na) ng = na;
+            if (ng < v && 2 * ng >= v) ng = (v + 1) / 2;     // two launches: equal ones
+            L.ng = (int)ng;
             if (L.ng > 1) {
                 const long long passes = at_end ? (L.ng + over - 1) / over : 1;
                 L.nr = (int)((L.ng + passes - 1) / passes);
-                L.Gpart = at_end ? (off - L.nr * part1) / 256 * 256 : L.Gblk + L.ng * g1;
+                L.Gpart = at_end ? (off - L.nr * part1) / 256 * 256 : L.KR64 + L.ng * g1;
                 L.part_dirty = at_end && L.Gpart < L.PART ? L.PART - L.Gpart : 0;
             } else {
                 L.ng = L.nr = 1;
@@ -1401,7 +1403,9 @@ int ppl_exact_contract_mixed(ppl_cpd* h, double* normR2, double* E_exact, double
     const int ng = h->L.ng;
     const long long pQ = (long long)v * v * pq.kX, bG = (long long)v * pq.kvv, pG = bG * ng;
     float* part = h->at<float>(ng > 1 ? h->L.Gpart : h->L.PART);
-    void* G = opb(h, ng > 1 ? h->L.Gblk : h->L.Gop);
+    void* G = opb(h, ng > 1 ? h->L.KR64 : h->L.Gop);
+    double* Rall = R_out ? R_out : h->at<double>(h->L.Rblk);
+    const bool whole = h->L.na >= v;      // (Rblk holds R) one reduction at the end, with R_out or without
     if (ng > 1)      // (Gop's K padding is zero as it is)
         zero_padding(h->opts.precision, G, pG, (long long)ng * v, v, v, pq.ldk, h->st);
     for (int a = 0; a < v && !e; a += ng) {
@@ -1417,7 +1421,7 @@ int ppl_exact_contract_mixed(ppl_cpd* h, double* normR2, double* E_exact, double
         e = run_tc(h, g1, "exact G");
         if (e) break;
         // R[a][b][ij] = sum_{cd} G_a[b][cd] tau[ij][cd], split-K summed in FP64
-        double* Rdst = R_out ? R_out + (long long)a * vo2 : h->at<double>(h->L.Rblk);
+        double* Rdst = Rall + (whole || R_out ? (long long)a * vo2 : 0);
         for (int b0 = 0; b0 < nb && !e; b0 += h->L.nr) {
             TcGemm g2{};
             g2.A = pmat(G, pG, v, (int)pq.kvv, nb, v, bG);
@@ -1427,9 +1431,9 @@ int ppl_exact_contract_mixed(ppl_cpd* h, double* normR2, double* E_exact, double
             g2.M = v; g2.N = o * o; g2.K = (int)pq.kvv; g2.batch = (nb - b0 < h->L.nr) ? nb - b0 : h->L.nr;
             e = run_tc_partial(h, g2, part, Rdst + b0 * vo2, (long long)o * o, vo2, "exact R");
         }
-        if (e) break;
-        exact_reduce(Rdst, a, nb, v, o, gov, h->at<double>(h->L.partial), acc, h->st);
+        if (!whole && !e) exact_reduce(Rdst, a, nb, v, o, gov, h->at<double>(h->L.partial), acc, h->st);
     }
+    if (whole && !e) exact_reduce(Rall, 0, v, v, o, gov, h->at<double>(h->L.partial), acc, h->st);
     // the intermediates' K padding reads as zero again
     if (h->L.part_dirty) zero_bytes(part, h->L.part_dirty, h->st);
     if (!e) e = check_cuda(h, "exact_contract_mixed");

@@ -35,8 +35,8 @@
 // tile extracts the rows that it shares with others again), with the MMAs (74 of
 // 128 x 64 x 16 per 32 values of k, 64 clocks each) under it, then the rounding and
 // writing of the tile.  Measured: an energy at o = 20, v = 200, X = 600, R = 800, two
-// contractions of M = 12000, N = 800, K = 200, 0.836 ms in all (0.851 with seven digits and
-// the rows' norms in place of their counts), 21.7 ms with k_gemm64 and 20-row tiles.
+// contractions of M = 12000, N = 800, K = 200, 0.857 ms in all (the same with seven digits
+// and the rows' norms in place of their counts), 21.7 ms with k_gemm64 and 20-row tiles.
 #include "ppl_internal.h"
 #include "ppl_gemm64.cuh"
 #include "ppl_ptx.cuh"

@@ -896,16 +896,16 @@ __global__ void __launch_bounds__(RPT) k_reduce_partials(const float* part, long
     out[(long long)blockIdx.y * ob + (long long)m * ldo + n] = s;
 }
 
-// The last npad columns of the last K panel (of ld columns) of each group.  Two planes of 17 x
-// 120 groups of 120 rows: 31 MB of sectors.
+// The last npad columns of the last K panel (of ld columns) of group blockIdx.x, plane
+// blockIdx.y, `rows` rows.  Bound by the writes, a part of a 128-byte row each (two planes of 51
+// x 70 groups of 70 rows x 26 columns: 52 MB).
 template <class T>
-__global__ void k_zero_padding(T* p, long long plane, long long groups, int rows, int ke, int npad, long long ld,
-                               long long total) {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
-        const int t = (int)(e % npad), b = (int)(e / npad % rows);
-        const long long g = e / npad / rows;          // (plane, group)
-        p[g / groups * plane + (g % groups * ld + ld - ke) * rows + (long long)b * ke + ke - npad + t] = T(0);
-    }
+__global__ void __launch_bounds__(256) k_zero_padding(T* p, long long plane, int rows, int ke, int npad, long long ld) {
+    T* q = p + blockIdx.y * plane + ((long long)blockIdx.x * ld + ld - ke) * rows + ke - npad;
+    const int per = 256 / npad;               // rows per pass
+    const int t = threadIdx.x % npad, b0 = threadIdx.x / npad;
+    if (b0 >= per) return;
+    for (int b = b0; b < rows; b += per) q[(long long)b * ke + t] = T(0);
 }
 
 // Batched transpose of operand planes: dst[b][j][i] = src[b][i][j] for i, j < n
@@ -1400,13 +1400,13 @@ void zero_bytes(void* p, size_t n, cudaStream_t s) {
 
 void zero_padding(int prec, void* p, long long plane_elems, long long groups, int rows, int cols, long long ld,
                   cudaStream_t s) {
-    const int ke = panel_width(prec), npad = (int)(ld - cols), planes = prec == PPL_PREC_TF32 ? 1 : 2;
-    const long long total = (long long)planes * groups * rows * npad;
-    if (total <= 0) return;
+    const int ke = panel_width(prec), npad = (int)(ld - cols);
+    if (npad <= 0 || groups <= 0 || rows <= 0) return;
+    const dim3 grid((unsigned)groups, prec == PPL_PREC_TF32 ? 1 : 2);
     if (prec == PPL_PREC_BF16X3)
-        k_zero_padding<<<grid_for(total, 256), 256, 0, s>>>((unsigned short*)p, plane_elems, groups, rows, ke, npad, ld, total);
+        k_zero_padding<<<grid, 256, 0, s>>>((unsigned short*)p, plane_elems, rows, ke, npad, ld);
     else
-        k_zero_padding<<<grid_for(total, 256), 256, 0, s>>>((unsigned int*)p, plane_elems, groups, rows, ke, npad, ld, total);
+        k_zero_padding<<<grid, 256, 0, s>>>((unsigned int*)p, plane_elems, rows, ke, npad, ld);
 }
 
 // ---- several captured contractions as one persistent launch ------------------
