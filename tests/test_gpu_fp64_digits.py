@@ -22,7 +22,9 @@ import pytest
 
 torch = pytest.importorskip("torch")
 
-from paper_2503_10380_gb300 import binding
+from oracle import ppl_oracle as orc
+from paper_2503_10380_gb300 import binding, inputs
+from parity import abs_factors, check_abs_bound
 
 pytestmark = pytest.mark.gpu
 
@@ -220,4 +222,43 @@ def test_wait_limit_holds_in_a_captured_sweep():
     for m, x in cp.factors().items():
         assert torch.allclose(x, first[m], rtol=1e-9, atol=1e-9 * float(first[m].abs().max()))
     assert cp.stats()["timeouts"] == 1
+    cp.close()
+
+
+@pytest.mark.parametrize("kind", ["zeros", "spread", "wide"])
+@pytest.mark.parametrize("shape", [(5, 24, 72, 48), (3, 33, 97, 9), (9, 40, 150, 130)])
+def test_every_layout_of_the_method(shape, kind):
+    """MTTKRPs, the exact contraction and the energy in FP64 on inputs that leave elements to
+    FP64 FMAs or have sums without terms, in each of the layouts the method contracts
+    (strided and compound k, split K with atomic sums, batches).  "zeros": nine in ten
+    entries of B and tau; "spread": auxiliary functions over 2^40, factors over 2^10;
+    "wide": the entries of B over 2^60.  Bound: 1e-12 of the same chain on absolute values
+    (four contractions of up to 6000 terms at 2^-53 each side)."""
+    o, v, X, R = shape
+    inp = inputs.make_inputs(o, v, X, R, seed=21)
+    rng = np.random.default_rng(3)
+    B, tau, U = inp.B.copy(), inp.tau.copy(), {m: x.copy() for m, x in inp.factors.items()}
+    if kind == "zeros":
+        mask = rng.random(B.shape) < 0.1
+        B *= mask | mask.transpose(0, 2, 1)
+        tau *= rng.random(tau.shape) < 0.1
+    elif kind == "spread":
+        B *= 2.0 ** rng.permutation(np.linspace(-20, 20, X))[:, None, None]
+        for m in U:
+            U[m] *= 2.0 ** rng.uniform(-5, 5, U[m].shape)
+    else:
+        s = rng.uniform(-30, 30, B.shape)
+        B *= 2.0 ** (0.5 * (s + s.transpose(0, 2, 1)))
+    Bvv, aB, at, aU = B[:, o:, o:], np.abs(B), np.abs(tau), abs_factors(U)
+    cp = binding.CpAls(torch.from_numpy(B).cuda(), torch.from_numpy(tau).cuda(), U, precision="fp64")
+    for m in orc.MODES:
+        check_abs_bound(cp.mttkrp(m).cpu().numpy(), orc.mttkrp(Bvv, tau, U, m), orc.mttkrp(aB[:, o:, o:], at, aU, m), 1e-12,
+                        f"{kind} {shape} mode {m}")
+    n2, E, Rt = cp.exact_contract(want_R=True)
+    check_abs_bound(Rt.cpu().numpy(), orc.ppl_tensor(Bvv, tau), orc.ppl_tensor(aB[:, o:, o:], at), 1e-12, f"{kind} {shape} R")
+    one = np.ones(R)
+    # with |a| + |b| in both virtual modes the direct and the exchange sum are alike, each at
+    # least the sum of the |terms| of either; their difference 2 x - x is x
+    scale = 3.0 * orc.energy_cp(aB, o, {**aU, "a": aU["a"] + aU["b"], "b": aU["a"] + aU["b"]}, one)
+    assert abs(cp.energy() - orc.energy_cp(B, o, U, one)) <= 1e-12 * scale
     cp.close()
