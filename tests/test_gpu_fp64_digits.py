@@ -130,6 +130,29 @@ def test_largest_digits():
     assert np.all(err <= 0.51 * np.spacing(np.abs(ex)))
 
 
+def test_largest_digits_over_many_folds():
+    """The same with K = o^2 = 576: T[r][c][d] = sum_ij U_i[i][r] U_j[j][r] tau[i][j][c][d], which the
+    MTTKRP of mode a passes on unchanged where B is the identity and U_b picks d = 0."""
+    o, v, X, R = 24, 17, 2, 9
+    plus = 0x7f7f7f7f7f7f
+    minus = 127 * 256 ** 5 - 128 * sum(256 ** k for k in range(5))
+    rows, cols = [plus, minus, -plus], [minus, plus, -minus, -plus]
+    B = np.zeros((X, o + v, o + v))
+    B[0, o:, o:] = np.eye(v)
+    tau = np.broadcast_to(np.array([float(cols[c % 4]) for c in range(v)])[:, None], (o, o, v, v))
+    fac = {"a": np.ones((v, R)), "b": np.zeros((v, R)), "j": np.ones((o, R)),
+           "i": np.broadcast_to(np.array([float(rows[r % 3]) for r in range(R)]), (o, R))}
+    fac["b"][0] = 1.0
+    cp = binding.CpAls(torch.from_numpy(B).cuda(), torch.from_numpy(tau.copy()).cuda(),
+                       {m: x.copy() for m, x in fac.items()}, precision="fp64")
+    M = cp.mttkrp("a").cpu().numpy()
+    cp.close()
+    for c in range(v):
+        for r in range(R):
+            exact = o * o * rows[r % 3] * cols[c % 4]
+            assert abs(int(M[c, r]) - exact) <= 0.51 * np.spacing(abs(float(exact))), (c, r)
+
+
 @pytest.mark.parametrize("kind", ["random", "halves", "one", "wide"])
 @pytest.mark.parametrize("K", [33, 200, 300])
 def test_rows_with_zeros(kind, K):
